@@ -591,7 +591,7 @@ int ch_mlp_forward(const float *weights, const int64_t *rows, uint64_t n, float 
         m.load(weights, st);
         DevBuf<float> x;
         x.alloc(n * 16);
-        rows_to_features(reinterpret_cast<const long long *>(rows), n, x.ptr, st);
+        rows_to_features(reinterpret_cast<const long long *>(rows), n, m.logs.ptr, x.ptr, st);
         m.infer(x.ptr, n, y_out, st);
         CH_CUDA_TRY(cudaStreamSynchronize(st));
     });

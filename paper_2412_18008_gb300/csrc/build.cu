@@ -1778,7 +1778,7 @@ __global__ void __launch_bounds__(256) k_witness_dense(WArgs a, Dense dn) {
 // and as transformed floats for the MLP; then ed_last[u] = P[u] and one more
 // rescoring is counted.
 __global__ void k_features(Dev d, const uint32_t *A, uint32_t nA, uint32_t r, long long *rows,
-                           float *x) {
+                           const float *tab, float *x) {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nA;
          i += gridDim.x * blockDim.x) {
         const uint32_t u = A[i];
@@ -1825,7 +1825,7 @@ __global__ void k_features(Dev d, const uint32_t *A, uint32_t nA, uint32_t r, lo
         }
         if (x) {
             float *xr = x + (uint64_t)i * 16;
-            for (int k = 0; k < 16; ++k) xr[k] = k < MLP_NIN ? feature_transform(f[k]) : 0.f;
+            for (int k = 0; k < 16; ++k) xr[k] = k < MLP_NIN ? feature_transform(f[k], tab) : 0.f;
         }
         d.ed_last[u] = ed;
         d.rescore[u] += 1;
@@ -2858,7 +2858,8 @@ void Builder::run_rounds() {
                 int32_t *plog = tracing ? trace_prio.ptr + trace_count : nullptr;
                 const int ga = grid_for(nA, 256, sms * 8);
                 if (tracing || learned) {
-                    k_features<<<ga, 256, 0, st>>>(d, A.ptr, nA, r, rows, learned ? fx.ptr : nullptr);
+                    k_features<<<ga, 256, 0, st>>>(d, A.ptr, nA, r, rows, learned ? mlp.logs.ptr : nullptr,
+                                                   learned ? fx.ptr : nullptr);
                     CH_CHECK_LAUNCH();
                 }
                 if (learned) {

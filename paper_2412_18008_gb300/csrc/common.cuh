@@ -208,6 +208,30 @@ __device__ __forceinline__ uint32_t warp_append(bool pred, uint32_t *counter) {
     return base + __popc(mask & ((1u << lane_id()) - 1u));
 }
 
+// Programmatic dependent launch: a kernel launched with launch_pdl may start
+// while the kernel before it on the stream still runs; pdl_wait() waits until
+// that one has finished and its writes are visible. Every such kernel calls it
+// (before it touches what an earlier kernel wrote), so the order of a chain
+// of them is that of ordinary launches. pdl_launch() lets the next one start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+void launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    CH_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...));
+    count_launch();
+}
+
 inline int grid_for(uint64_t work, int block, int max_blocks) {
     uint64_t g = (work + block - 1) / block;
     if (g < 1) g = 1;

@@ -18,6 +18,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 
 #include "mlp.cuh"
 
@@ -158,97 +159,315 @@ k_mlp_infer(const float *x, uint64_t rows, const MlpFrag *fg, float *y) {
 
 constexpr int TR_THREADS = 256;
 
-// Per sample: transformed features x (16, 12 used), the forward pass with
-// the inference's roundings (inputs, W1, W2 and the first hidden layer in
-// BF16; W3, biases, the second hidden layer and the output in FP32), and the
-// backward pass down to the pre-activation gradients of both hidden layers.
+// Both training kernels keep every sum in the order one thread would take it
+// (k, j or the sample ascending, one fused multiply-add a term), so the
+// weights do not depend on how the work is split over threads.
+
+constexpr uint32_t TR_ROWS = 64;  // samples per forward / backward block
+constexpr int TR_PITCH = 68;      // row pitch of the 64-wide tiles (16-byte aligned, no bank conflicts)
+
+struct alignas(16) TrFwdSmem {  // every tile starts on 16 bytes (tr_tile's loads)
+    float w1[NIN][TR_PITCH];
+    float w2[NH][TR_PITCH];   // [k][j]
+    float w2t[NH][TR_PITCH];  // [j][k]
+    float xt[NIN][TR_PITCH];  // [k][sample]
+    float h1t[NH][TR_PITCH];  // [j][sample]
+    float h2t[NH][TR_PITCH];  // [j][sample], then the second layer's gradients
+    float b1[NH], b2[NH], w3[NH], dy[TR_ROWS];
+    float b3;
+};
+static_assert(TR_PITCH % 4 == 0, "rows of the tiles start on 16 bytes");
+static_assert(offsetof(TrFwdSmem, w2) % 16 == 0 && offsetof(TrFwdSmem, w2t) % 16 == 0 &&
+                  offsetof(TrFwdSmem, xt) % 16 == 0 && offsetof(TrFwdSmem, h1t) % 16 == 0 &&
+                  offsetof(TrFwdSmem, h2t) % 16 == 0,
+              "tiles start on 16 bytes");
+
+// acc[a][b] += p[k][4 * pa + a] * q[k][4 * qb + b] over k ascending.
+template <int K>
+__device__ __forceinline__ void tr_tile(float (&acc)[4][4], const float (*p)[TR_PITCH], uint32_t pa,
+                                        const float (*q)[TR_PITCH], uint32_t qb) {
+#pragma unroll 8
+    for (int k = 0; k < K; ++k) {
+        const float4 u = *reinterpret_cast<const float4 *>(&p[k][4 * pa]);
+        const float4 v = *reinterpret_cast<const float4 *>(&q[k][4 * qb]);
+        const float uu[4] = {u.x, u.y, u.z, u.w}, vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(uu[x], vv[y], acc[x][y]);
+    }
+}
+
+// Forward pass with the inference's roundings (inputs, W1, W2 and the first
+// hidden layer in BF16; W3, biases, the second hidden layer and the output in
+// FP32), and the backward pass down to the pre-activation gradients of both
+// hidden layers, for 64 samples a block. Each product with a weight matrix is
+// a 64 x 64 tile in which a thread keeps 4 x 4 outputs in registers and reads
+// its operands from shared memory, two 16-byte loads for 16 multiply-adds
+// (a thread a sample, its layers in local memory, took 80 us for 8192
+// samples; this takes 18).
 __global__ void __launch_bounds__(TR_THREADS)
 k_train_fwd_bwd(const float *x, const float *label, uint64_t b0, uint32_t bsz, const float *wq,
-                float *h1o, float *h2o, float *g1o, float *g2o, float *dyo, float *loss_part) {
-    __shared__ float W[MLP_NPARAM];
-    for (uint32_t i = threadIdx.x; i < (uint32_t)MLP_NPARAM; i += blockDim.x) W[i] = wq[i];
+                float *h1o, float *h2o, float *g1o, float *g2o, float *dyo, float *loss_sq) {
+    extern __shared__ __align__(16) unsigned char tr_raw[];
+    TrFwdSmem &s = *reinterpret_cast<TrFwdSmem *>(tr_raw);
+    const uint32_t tid = threadIdx.x, tj = tid % 16, ts = tid / 16;
+    const uint32_t i0 = blockIdx.x * TR_ROWS;
+    // the inputs do not depend on the launch before this one
+    for (uint32_t t = tid; t < TR_ROWS * NIN; t += TR_THREADS) {
+        const uint32_t i = t / NIN, k = t % NIN;
+        s.xt[k][i] = i0 + i < bsz ? bf16_round(x[(b0 + i0 + i) * 16 + k]) : 0.f;
+    }
+    pdl_wait();
+    pdl_launch();
+    for (uint32_t t = tid; t < (uint32_t)(NIN * NH); t += TR_THREADS) s.w1[t / NH][t % NH] = wq[OFF_W1 + t];
+    for (uint32_t t = tid; t < (uint32_t)(NH * NH); t += TR_THREADS) {
+        const float w = wq[OFF_W2 + t];
+        s.w2[t / NH][t % NH] = w;
+        s.w2t[t % NH][t / NH] = w;
+    }
+    if (tid < (uint32_t)NH) {
+        s.b1[tid] = wq[OFF_B1 + tid];
+        s.b2[tid] = wq[OFF_B2 + tid];
+        s.w3[tid] = wq[OFF_W3 + tid];
+    }
+    if (tid == 0) s.b3 = wq[OFF_B3];
     __syncthreads();
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    float lsum = 0.f;
-    if (i < bsz) {
-        const uint64_t r = b0 + i;
-        float xi[NIN];
+    float acc[4][4];  // [sample][output]
 #pragma unroll
-        for (int k = 0; k < NIN; ++k) xi[k] = bf16_round(x[r * 16 + k]);
-        float h1[NH], h2[NH];
-        for (int j = 0; j < NH; ++j) {
-            float s = W[OFF_B1 + j];
+    for (int c = 0; c < 4; ++c)
 #pragma unroll
-            for (int k = 0; k < NIN; ++k) s += xi[k] * W[OFF_W1 + k * NH + j];
-            h1[j] = bf16_round(fmaxf(s, 0.f));
+        for (int o = 0; o < 4; ++o) acc[c][o] = s.b1[4 * tj + o];
+    tr_tile<NIN>(acc, s.xt, ts, s.w1, tj);
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s.h1t[4 * tj + o][4 * ts + c] = bf16_round(fmaxf(acc[c][o], 0.f));
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) acc[c][o] = s.b2[4 * tj + o];
+    tr_tile<NH>(acc, s.h1t, ts, s.w2, tj);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t i = i0 + 4 * ts + c;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            acc[c][o] = fmaxf(acc[c][o], 0.f);
+            s.h2t[4 * tj + o][4 * ts + c] = acc[c][o];
         }
-        for (int j = 0; j < NH; ++j) {
-            float s = W[OFF_B2 + j];
-            for (int k = 0; k < NH; ++k) s += h1[k] * W[OFF_W2 + k * NH + j];
-            h2[j] = fmaxf(s, 0.f);
+        if (i < bsz)
+            *reinterpret_cast<float4 *>(h2o + (uint64_t)i * NH + 4 * tj) =
+                make_float4(acc[c][0], acc[c][1], acc[c][2], acc[c][3]);
+    }
+    __syncthreads();
+    if (tid < TR_ROWS) {
+        const uint32_t i = i0 + tid;
+        float y = s.b3;
+#pragma unroll 16
+        for (int j = 0; j < NH; ++j) y = fmaf(s.h2t[j][tid], s.w3[j], y);
+        float dy = 0.f;
+        if (i < bsz) {
+            const float diff = y - label[b0 + i];
+            loss_sq[i] = diff * diff;
+            dy = 2.f * diff / (float)bsz;
+            dyo[i] = dy;
         }
-        float y = W[OFF_B3];
-        for (int j = 0; j < NH; ++j) y += h2[j] * W[OFF_W3 + j];
-        const float diff = y - label[r];
-        lsum = diff * diff;
-        const float dy = 2.f * diff / (float)bsz;
-        dyo[i] = dy;
-        float g2[NH];
-        for (int j = 0; j < NH; ++j) {
-            g2[j] = h2[j] > 0.f ? dy * W[OFF_W3 + j] : 0.f;
-            h1o[(uint64_t)i * NH + j] = h1[j];
-            h2o[(uint64_t)i * NH + j] = h2[j];
-            g2o[(uint64_t)i * NH + j] = g2[j];
+        s.dy[tid] = dy;
+    }
+    __syncthreads();
+    // the second layer's gradients: this thread's own 4 x 4 outputs
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t i = i0 + 4 * ts + c;
+        float g[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            g[o] = acc[c][o] > 0.f ? s.dy[4 * ts + c] * s.w3[4 * tj + o] : 0.f;
+            s.h2t[4 * tj + o][4 * ts + c] = g[o];
+            acc[c][o] = 0.f;
         }
-        for (int k = 0; k < NH; ++k) {
-            float s = 0.f;
-            for (int j = 0; j < NH; ++j) s += g2[j] * W[OFF_W2 + k * NH + j];
-            g1o[(uint64_t)i * NH + k] = h1[k] > 0.f ? s : 0.f;
+        if (i < bsz)
+            *reinterpret_cast<float4 *>(g2o + (uint64_t)i * NH + 4 * tj) = make_float4(g[0], g[1], g[2], g[3]);
+    }
+    __syncthreads();
+    tr_tile<NH>(acc, s.h2t, ts, s.w2t, tj);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t i = i0 + 4 * ts + c;
+        if (i >= bsz) continue;
+        float h[4], g[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            h[o] = s.h1t[4 * tj + o][4 * ts + c];
+            g[o] = h[o] > 0.f ? acc[c][o] : 0.f;
+        }
+        *reinterpret_cast<float4 *>(h1o + (uint64_t)i * NH + 4 * tj) = make_float4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<float4 *>(g1o + (uint64_t)i * NH + 4 * tj) = make_float4(g[0], g[1], g[2], g[3]);
+    }
+}
+
+constexpr uint32_t TR_SLICE = 512;    // samples per partial-gradient sum
+constexpr uint32_t TR_CHUNK = 64;     // samples staged at a time
+constexpr uint32_t TR_PARTS = 10;     // parameter groups: W2 by 8 rows (with b2 in the first), W1 + b1, W3 + b3
+constexpr int TRG_THREADS = 128;
+constexpr uint32_t TR_STAGES = 4;     // chunks in shared memory: 64 columns of one operand, up to 16 of the other
+constexpr int TRG_SMEM = TR_STAGES * TR_CHUNK * (NH + 16) * (int)sizeof(float);
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
+// Partial gradients over a slice of 512 samples, each parameter's sum taken in
+// sample order by one thread. A block takes one slice and one group of
+// parameters and streams both operands through a ring of four chunks of 64
+// samples (asynchronous copies, 80 KB, so that two blocks share an SM and the
+// 160 blocks of 8192 samples run at once); a thread holds 2 x 2 sums of W2
+// (or 4 x 2 of W1), so that its chains hide each other's latency. Bound by the
+// chain of 512 dependent multiply-adds and the staging. (One block a slice, a
+// thread a parameter reading global memory: 16 blocks and 470 us for 8192
+// samples; this takes 22.)
+__global__ void __launch_bounds__(TRG_THREADS)
+k_train_grad_part(const float *x, uint64_t b0, uint32_t bsz, const float *h1, const float *h2,
+                  const float *g1, const float *g2, const float *dy, float *part) {
+    extern __shared__ __align__(16) unsigned char tr_raw[];
+    float(*sa)[NH] = reinterpret_cast<float(*)[NH]>(tr_raw);  // [ring position][64]
+    float(*sb)[16] = reinterpret_cast<float(*)[16]>(tr_raw + TR_STAGES * TR_CHUNK * NH * sizeof(float));
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t s0 = blockIdx.x * TR_SLICE, ns = min(bsz - s0, TR_SLICE);
+    const uint32_t grp = blockIdx.y;
+    float *out = part + (uint64_t)blockIdx.x * MLP_NPARAM;
+    const float *wide = grp < 8 ? g2 : (grp == 8 ? g1 : h2);
+    const uint32_t nchunk = (ns + TR_CHUNK - 1) / TR_CHUNK;
+    auto stage = [&](uint32_t c) {
+        if (c < nchunk) {
+            const uint32_t i0 = c * TR_CHUNK, m = min(ns - i0, TR_CHUNK), r0 = (c % TR_STAGES) * TR_CHUNK;
+            for (uint32_t t = tid; t < m * (NH / 4); t += TRG_THREADS) {
+                const uint32_t i = t / (NH / 4), q = 4 * (t % (NH / 4));
+                cp_async16(&sa[r0 + i][q], wide + (uint64_t)(s0 + i0 + i) * NH + q);
+            }
+            if (grp < 8) {  // 8 columns of the first hidden layer
+                for (uint32_t t = tid; t < m * 2; t += TRG_THREADS) {
+                    const uint32_t i = t / 2, q = 4 * (t % 2);
+                    cp_async16(&sb[r0 + i][q], h1 + (uint64_t)(s0 + i0 + i) * NH + 8 * grp + q);
+                }
+            } else if (grp == 8) {  // the inputs
+                for (uint32_t t = tid; t < m * 4; t += TRG_THREADS) {
+                    const uint32_t i = t / 4, q = 4 * (t % 4);
+                    cp_async16(&sb[r0 + i][q], x + (b0 + s0 + i0 + i) * 16 + q);
+                }
+            } else {
+                for (uint32_t i = tid; i < m; i += TRG_THREADS) cp_async4(&sb[r0 + i][0], dy + s0 + i0 + i);
+            }
+        }
+        cp_async_commit();  // one group a chunk, empty past the last
+    };
+    pdl_wait();
+    pdl_launch();
+    for (uint32_t c = 0; c + 1 < TR_STAGES; ++c) stage(c);
+    const uint32_t j = 2 * lane;
+    float acc[4][2] = {}, ones[2] = {};
+    for (uint32_t c = 0; c < nchunk; ++c) {
+        cp_async_wait<TR_STAGES - 2>();
+        __syncthreads();  // chunk c has arrived, chunk c - 1 is used up
+        stage(c + TR_STAGES - 1);
+        const uint32_t i0 = (c % TR_STAGES) * TR_CHUNK, i1 = i0 + min(ns - c * TR_CHUNK, TR_CHUNK);
+        if (grp < 8) {
+            // rows 8 * grp + 2 * warp and the next one of W2
+#pragma unroll 8
+            for (uint32_t i = i0; i < i1; ++i) {
+                const float2 g = *reinterpret_cast<const float2 *>(&sa[i][j]);
+                const float2 h = *reinterpret_cast<const float2 *>(&sb[i][2 * warp]);
+                acc[0][0] = fmaf(h.x, g.x, acc[0][0]);
+                acc[0][1] = fmaf(h.x, g.y, acc[0][1]);
+                acc[1][0] = fmaf(h.y, g.x, acc[1][0]);
+                acc[1][1] = fmaf(h.y, g.y, acc[1][1]);
+                ones[0] += g.x;
+                ones[1] += g.y;
+            }
+        } else if (grp == 8) {
+            // rows 4 * warp .. 4 * warp + 3 of W1 for the first three warps, b1 for the last
+#pragma unroll 8
+            for (uint32_t i = i0; i < i1; ++i) {
+                const float2 g = *reinterpret_cast<const float2 *>(&sa[i][j]);
+                const float4 v = *reinterpret_cast<const float4 *>(&sb[i][4 * warp]);
+                const float vv[4] = {bf16_round(v.x), bf16_round(v.y), bf16_round(v.z), bf16_round(v.w)};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    acc[q][0] = fmaf(vv[q], g.x, acc[q][0]);
+                    acc[q][1] = fmaf(vv[q], g.y, acc[q][1]);
+                }
+                ones[0] += g.x;
+                ones[1] += g.y;
+            }
+        } else if (warp == 0) {
+#pragma unroll 8
+            for (uint32_t i = i0; i < i1; ++i) {
+                const float2 h = *reinterpret_cast<const float2 *>(&sa[i][j]);
+                const float v = sb[i][0];
+                acc[0][0] = fmaf(h.x, v, acc[0][0]);
+                acc[0][1] = fmaf(h.y, v, acc[0][1]);
+                ones[0] += v;
+            }
         }
     }
-    // block sum of the squared errors, in a fixed order
+    if (grp < 8) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            float *o = out + OFF_W2 + (8 * grp + 2 * warp + q) * NH + j;
+            o[0] = acc[q][0];
+            o[1] = acc[q][1];
+        }
+        if (grp == 0 && warp == 0) {
+            out[OFF_B2 + j] = ones[0];
+            out[OFF_B2 + j + 1] = ones[1];
+        }
+    } else if (grp == 8) {
+        if (warp < 3) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float *o = out + OFF_W1 + (4 * warp + q) * NH + j;
+                o[0] = acc[q][0];
+                o[1] = acc[q][1];
+            }
+        } else {
+            out[OFF_B1 + j] = ones[0];
+            out[OFF_B1 + j + 1] = ones[1];
+        }
+    } else if (warp == 0) {
+        out[OFF_W3 + j] = acc[0][0];
+        out[OFF_W3 + j + 1] = acc[0][1];
+        if (lane == 0) out[OFF_B3] = ones[0];
+    }
+}
+
+// Sums of the squared errors over 256 samples of a minibatch each, by a fixed
+// tree: block p of minibatch q (of bsz samples, per_batch blocks) of n samples.
+__global__ void __launch_bounds__(TR_THREADS)
+k_train_loss(const float *sq, uint64_t n, uint32_t bsz, uint32_t per_batch, float *out) {
     __shared__ float red[TR_THREADS];
-    red[threadIdx.x] = lsum;
+    const uint64_t m0 = (uint64_t)(blockIdx.x / per_batch) * bsz;
+    const uint64_t left = n - m0;
+    const uint32_t mb = left < bsz ? (uint32_t)left : bsz;
+    const uint32_t i = (blockIdx.x % per_batch) * TR_THREADS + threadIdx.x;
+    red[threadIdx.x] = i < mb ? sq[m0 + i] : 0.f;
     __syncthreads();
-    for (uint32_t st = blockDim.x / 2; st > 0; st >>= 1) {
+    for (uint32_t st = TR_THREADS / 2; st > 0; st >>= 1) {
         if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
         __syncthreads();
     }
-    if (threadIdx.x == 0) loss_part[blockIdx.x] = red[0];
-}
-
-constexpr uint32_t TR_SLICE = 512;  // samples per partial-gradient block
-
-// Partial gradients over a slice of samples: one thread per parameter
-// group, summing the slice in sample order.
-__global__ void __launch_bounds__(TR_THREADS)
-k_train_grad_part(const float *x, uint64_t b0, uint32_t bsz, const float *h1, const float *h2,
-                  const float *g1, const float *g2, const float *dy, float *part) {
-    const uint32_t s0 = blockIdx.x * TR_SLICE;
-    const uint32_t s1 = min(bsz, s0 + TR_SLICE);
-    float *out = part + (uint64_t)blockIdx.x * MLP_NPARAM;
-    for (uint32_t p = threadIdx.x; p < (uint32_t)MLP_NPARAM; p += blockDim.x) {
-        float s = 0.f;
-        if (p < (uint32_t)OFF_B1) {  // W1[k][j] += x_k * g1_j
-            const uint32_t k = p / NH, j = p % NH;
-            for (uint32_t i = s0; i < s1; ++i) s += bf16_round(x[(b0 + i) * 16 + k]) * g1[(uint64_t)i * NH + j];
-        } else if (p < (uint32_t)OFF_W2) {
-            const uint32_t j = p - OFF_B1;
-            for (uint32_t i = s0; i < s1; ++i) s += g1[(uint64_t)i * NH + j];
-        } else if (p < (uint32_t)OFF_B2) {  // W2[k][j] += h1_k * g2_j
-            const uint32_t k = (p - OFF_W2) / NH, j = (p - OFF_W2) % NH;
-            for (uint32_t i = s0; i < s1; ++i) s += h1[(uint64_t)i * NH + k] * g2[(uint64_t)i * NH + j];
-        } else if (p < (uint32_t)OFF_W3) {
-            const uint32_t j = p - OFF_B2;
-            for (uint32_t i = s0; i < s1; ++i) s += g2[(uint64_t)i * NH + j];
-        } else if (p < (uint32_t)OFF_B3) {  // W3[j] += h2_j * dy
-            const uint32_t j = p - OFF_W3;
-            for (uint32_t i = s0; i < s1; ++i) s += h2[(uint64_t)i * NH + j] * dy[i];
-        } else {
-            for (uint32_t i = s0; i < s1; ++i) s += dy[i];
-        }
-        out[p] = s;
-    }
+    if (threadIdx.x == 0) out[blockIdx.x] = red[0];
 }
 
 // grad[p] = sum of the partials in slice order; then Adam on the FP32
@@ -256,9 +475,12 @@ k_train_grad_part(const float *x, uint64_t b0, uint32_t bsz, const float *h1, co
 __global__ void k_train_adam(const float *part, uint32_t nparts, float *grad, float *w, float *wq,
                              float *m, float *v, float lr, float b1, float b2, float eps,
                              float b1t, float b2t, int apply) {
+    pdl_wait();
+    pdl_launch();
     for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < (uint32_t)MLP_NPARAM;
          p += gridDim.x * blockDim.x) {
         float g = 0.f;
+#pragma unroll 16
         for (uint32_t k = 0; k < nparts; ++k) g += part[(uint64_t)k * MLP_NPARAM + p];
         grad[p] = g;
         if (!apply) continue;
@@ -279,12 +501,17 @@ __global__ void k_round_weights(const float *w, float *wq) {
         wq[p] = quantised(p, w[p]);
 }
 
+__global__ void k_log_table(float *tab) {
+    const uint32_t a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a < LOG_TAB) tab[a] = feature_transform((long long)a);
+}
+
 // Transformed features of trace rows (round, vertex, 12 features).
-__global__ void k_rows_to_x(const long long *rows, uint64_t n, float *x) {
+__global__ void k_rows_to_x(const long long *rows, uint64_t n, const float *tab, float *x) {
     for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < n;
          r += (uint64_t)gridDim.x * blockDim.x) {
 #pragma unroll
-        for (int k = 0; k < 16; ++k) x[r * 16 + k] = k < NIN ? feature_transform(rows[r * 14 + 2 + k]) : 0.f;
+        for (int k = 0; k < 16; ++k) x[r * 16 + k] = k < NIN ? feature_transform(rows[r * 14 + 2 + k], tab) : 0.f;
     }
 }
 
@@ -313,6 +540,8 @@ MlpDevice::~MlpDevice() = default;
 void MlpDevice::load(const float *host_weights, cudaStream_t st) {
     weights.alloc(MLP_NPARAM);
     frag.alloc((sizeof(MlpFrag) + 3) / 4);
+    logs.alloc(LOG_TAB);
+    log_table(logs.ptr, st);
     CH_CUDA_TRY(cudaMemcpyAsync(weights.ptr, host_weights, MLP_NPARAM * sizeof(float),
                                 cudaMemcpyHostToDevice, st));
     k_mlp_prepare<<<1, 256, 0, st>>>(weights.ptr, reinterpret_cast<MlpFrag *>(frag.ptr));
@@ -326,17 +555,24 @@ void MlpDevice::infer(const float *x, uint64_t rows, float *y, cudaStream_t st) 
     CH_CHECK_LAUNCH();
 }
 
-void rows_to_features(const long long *rows, uint64_t n, float *x, cudaStream_t st) {
+void log_table(float *tab, cudaStream_t st) {
+    k_log_table<<<LOG_TAB / 64, 64, 0, st>>>(tab);
+    CH_CHECK_LAUNCH();
+}
+
+void rows_to_features(const long long *rows, uint64_t n, const float *tab, float *x, cudaStream_t st) {
     if (!n) return;
-    k_rows_to_x<<<grid_for(n, 256, device_sm_count() * 8), 256, 0, st>>>(rows, n, x);
+    k_rows_to_x<<<grid_for(n, 256, device_sm_count() * 8), 256, 0, st>>>(rows, n, tab, x);
     CH_CHECK_LAUNCH();
 }
 
 void mlp_train(const long long *rows, const float *labels, uint64_t n, const ch_train_params_t *tp,
                float *weights_io, float *loss_out, float *grad_out, cudaStream_t st) {
-    DevBuf<float> x, w, wq, m, v, grad, h1, h2, g1, g2, dy, part, lpart;
+    DevBuf<float> logs, x, w, wq, m, v, grad, h1, h2, g1, g2, dy, part, sq, lpart;
+    logs.alloc(LOG_TAB);
+    log_table(logs.ptr, st);
     x.alloc(n * 16);
-    rows_to_features(rows, n, x.ptr, st);
+    rows_to_features(rows, n, logs.ptr, x.ptr, st);
     w.alloc(MLP_NPARAM);
     wq.alloc(MLP_NPARAM);
     m.alloc(MLP_NPARAM);
@@ -355,36 +591,41 @@ void mlp_train(const long long *rows, const float *labels, uint64_t n, const ch_
     dy.alloc(B);
     const uint32_t nparts = (B + TR_SLICE - 1) / TR_SLICE;
     part.alloc((uint64_t)nparts * MLP_NPARAM);
-    const uint32_t fb_blocks = (B + TR_THREADS - 1) / TR_THREADS;
-    lpart.alloc(fb_blocks);
-    std::vector<float> hl(fb_blocks);
     float b1t = 1.f, b2t = 1.f;
     const bool apply = tp->epochs > 0;
     const uint32_t epochs = apply ? tp->epochs : 1;
+    const uint64_t seen = apply ? n : B;  // samples an epoch goes over
+    // squared errors of an epoch, summed and read back once at its end: no
+    // step waits for the host
+    const uint32_t per_batch = (B + TR_THREADS - 1) / TR_THREADS;
+    const uint64_t lblocks = (seen + B - 1) / B * per_batch;
+    if (lblocks > 0x7FFFFFFFull) throw Error{CH_ERANGE, "too many minibatches"};
+    sq.alloc(seen);
+    lpart.alloc(lblocks);
+    std::vector<float> hl(lblocks);
+    CH_CUDA_TRY(cudaFuncSetAttribute(k_train_fwd_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(TrFwdSmem)));
+    CH_CUDA_TRY(cudaFuncSetAttribute(k_train_grad_part, cudaFuncAttributeMaxDynamicSharedMemorySize, TRG_SMEM));
     for (uint32_t ep = 0; ep < epochs; ++ep) {
         double ep_loss = 0;
-        for (uint64_t b0 = 0; b0 < n; b0 += B) {
+        for (uint64_t b0 = 0; b0 < seen; b0 += B) {
             const uint32_t bsz = (uint32_t)std::min<uint64_t>(B, n - b0);
-            const uint32_t fbb = (bsz + TR_THREADS - 1) / TR_THREADS;
-            k_train_fwd_bwd<<<fbb, TR_THREADS, 0, st>>>(x.ptr, labels, b0, bsz, wq.ptr, h1.ptr,
-                                                        h2.ptr, g1.ptr, g2.ptr, dy.ptr, lpart.ptr);
-            CH_CHECK_LAUNCH();
+            launch_pdl(k_train_fwd_bwd, (bsz + TR_ROWS - 1) / TR_ROWS, TR_THREADS, sizeof(TrFwdSmem), st, x.ptr,
+                       labels, b0, bsz, wq.ptr, h1.ptr, h2.ptr, g1.ptr, g2.ptr, dy.ptr, sq.ptr + b0);
             const uint32_t np = (bsz + TR_SLICE - 1) / TR_SLICE;
-            k_train_grad_part<<<np, TR_THREADS, 0, st>>>(x.ptr, b0, bsz, h1.ptr, h2.ptr, g1.ptr,
-                                                         g2.ptr, dy.ptr, part.ptr);
-            CH_CHECK_LAUNCH();
+            launch_pdl(k_train_grad_part, dim3(np, TR_PARTS), TRG_THREADS, TRG_SMEM, st, x.ptr, b0, bsz, h1.ptr,
+                       h2.ptr, g1.ptr, g2.ptr, dy.ptr, part.ptr);
             b1t *= tp->beta1;
             b2t *= tp->beta2;
-            k_train_adam<<<20, 256, 0, st>>>(part.ptr, np, grad.ptr, w.ptr, wq.ptr, m.ptr, v.ptr,
-                                              tp->lr, tp->beta1, tp->beta2, tp->eps, b1t, b2t,
-                                              apply ? 1 : 0);
-            CH_CHECK_LAUNCH();
-            CH_CUDA_TRY(cudaMemcpyAsync(hl.data(), lpart.ptr, fbb * 4, cudaMemcpyDeviceToHost, st));
-            CH_CUDA_TRY(cudaStreamSynchronize(st));
-            for (uint32_t k = 0; k < fbb; ++k) ep_loss += hl[k];
-            if (!apply) break;  // gradient of the first batch only
+            launch_pdl(k_train_adam, 20, 256, 0, st, part.ptr, np, grad.ptr, w.ptr, wq.ptr, m.ptr, v.ptr, tp->lr,
+                       tp->beta1, tp->beta2, tp->eps, b1t, b2t, apply ? 1 : 0);
         }
-        if (loss_out) loss_out[ep] = (float)(ep_loss / (double)(apply ? n : std::min<uint64_t>(B, n)));
+        k_train_loss<<<(unsigned)lblocks, TR_THREADS, 0, st>>>(sq.ptr, seen, B, per_batch, lpart.ptr);
+        CH_CHECK_LAUNCH();
+        CH_CUDA_TRY(cudaMemcpyAsync(hl.data(), lpart.ptr, lblocks * 4, cudaMemcpyDeviceToHost, st));
+        CH_CUDA_TRY(cudaStreamSynchronize(st));
+        for (const float l : hl) ep_loss += l;
+        if (loss_out) loss_out[ep] = (float)(ep_loss / (double)seen);
     }
     if (apply)
         CH_CUDA_TRY(cudaMemcpyAsync(weights_io, w.ptr, MLP_NPARAM * 4, cudaMemcpyDeviceToDevice, st));

@@ -17,11 +17,27 @@ __host__ __device__ __forceinline__ float feature_transform(long long x) {
     return x < 0 ? -v : v;
 }
 
+// The transform through a table of its values at |x| < LOG_TAB (log_table's):
+// a double-precision logarithm costs about a microsecond on this chip, and
+// nearly all features are small. Same bits either way.
+constexpr uint32_t LOG_TAB = 4096;
+
+__device__ __forceinline__ float feature_transform(long long x, const float *tab) {
+    const unsigned long long a = x < 0 ? 0ull - (unsigned long long)x : (unsigned long long)x;
+    if (a >= LOG_TAB) return feature_transform(x);
+    const float v = __ldg(tab + a);
+    return x < 0 ? -v : v;
+}
+
+// Fills tab[LOG_TAB].
+void log_table(float *tab, cudaStream_t st);
+
 // Weights resident on the device: FP32 copy and the BF16 tensor-core
 // fragments of W1 and W2.
 struct MlpDevice {
     DevBuf<float> weights;
     DevBuf<uint32_t> frag;
+    DevBuf<float> logs;  // feature_transform's table
     MlpDevice();
     ~MlpDevice();
     void load(const float *host_weights, cudaStream_t st);
@@ -29,8 +45,9 @@ struct MlpDevice {
     void infer(const float *x, uint64_t rows, float *y, cudaStream_t st) const;
 };
 
-// x[r] = transformed features of trace rows (round, vertex, 12 features).
-void rows_to_features(const long long *rows, uint64_t n, float *x, cudaStream_t st);
+// x[r] = transformed features of trace rows (round, vertex, 12 features); tab
+// is log_table's.
+void rows_to_features(const long long *rows, uint64_t n, const float *tab, float *x, cudaStream_t st);
 
 // y[r] = training target of trace row r: sign(x) * log2(1 + |x|) of
 // x = edge difference + 2 * hierarchy depth at that rescoring.

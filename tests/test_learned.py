@@ -258,6 +258,27 @@ def test_mlp_forward_and_gradient_match_cpu_reference():
 
 
 @gpu
+@pytest.mark.parametrize("count", [1, 63, 64, 65, 511, 513, 1025])
+def test_gradient_at_ragged_batch_sizes(count):
+    """Edges of the 64-sample blocks and chunks and of the 512-sample slices,
+    with the bound of the test above."""
+    torch = _torch()
+    ch = _ch()
+    rows, labels = _train_data([I.geometric_knn_graph(2_000, seed=52)])
+    rows, labels = rows[:count], labels[:count]
+    w = M.init_weights(3)
+    X = M.transform(rows[:, 2:])
+    dw = torch.from_numpy(w.copy()).cuda()
+    grad, loss = ch.mlp_train(torch.from_numpy(rows).cuda(), torch.from_numpy(labels).cuda(), dw, epochs=0,
+                              batch=count)
+    L_ref, g_ref = M.loss_and_grad(w, X, labels.astype(np.float64))
+    g = grad.cpu().numpy().astype(np.float64)
+    bound = grad_error_bound(w, X, labels)
+    bad = np.nonzero(np.abs(g - g_ref) > bound)[0]
+    assert bad.size == 0, (bad[:10], g[bad[:10]], g_ref[bad[:10]], bound[bad[:10]])
+
+
+@gpu
 def test_training_lowers_loss_and_is_deterministic():
     torch = _torch()
     ch = _ch()
