@@ -58,8 +58,8 @@ struct QArgs {
     // Work items and counters. A block kernel takes items from work[ctr]:
     // query j for j < k, or, with in_list, query in_list[j] for
     // j < work[in_cnt]. A query whose search overflows is appended to ovf,
-    // counted in work[ovf_cnt]. The dense kernel takes ovf entries from
-    // work[1].
+    // counted in work[ovf_cnt]. The dense kernel takes ovf entries (or, with
+    // dense_first, all queries) from work[1].
     uint32_t *work;
     const uint32_t *in_list;
     uint32_t in_cnt, ctr, ovf_cnt;
@@ -71,6 +71,11 @@ struct QArgs {
     // core_n distances) instead.
     const uint32_t *core_tab = nullptr;
     uint32_t core_lo = 0, core_n = 0;
+    // Dense kernel: first rank of the core (n without one), the bucket width
+    // its searches start with, and whether it takes every query of the batch
+    // instead of the overflowed ones.
+    uint32_t core_first = INF, dense_delta = 1;
+    bool dense_first = false;
     // Bucket width of delta-stepping levels (the DELTA kernels): a level
     // expands only the entries whose label is at most the least queued
     // label of their direction plus delta and keeps the rest queued.

@@ -13,7 +13,8 @@
 // shared-memory hash table whose entries carry both directions' distances,
 // so the meeting minimum is one pass over the table. A query whose search
 // spaces do not fit is redone by a second kernel that keeps labels in dense
-// per-vertex arrays in global memory (one block per array slot).
+// per-vertex arrays in global memory (one block per array slot); so is every
+// query of a hierarchy with a core that no table would hold.
 
 #include <algorithm>
 #include <mutex>
@@ -78,122 +79,263 @@ __global__ void __launch_bounds__(QB_THREADS, (STALL || DELTA) ? 6 : 1) k_query_
     qb_flush_stat(stat, a.stats);
 }
 
-// Dense fallback: one block per slot; labels in per-vertex arrays.
+// Queries on per-vertex label arrays in global memory (no capacity limit),
+// one block per slot: those that overflow the shared tables, and every query
+// of a hierarchy whose core is larger than a table (dense_first).
 struct QDense {
-    uint32_t *df, *db, *fst, *fa, *fb, *touched;
+    uint32_t *df, *db;   // labels, INF between queries
+    uint32_t *queued;    // bit d: the vertex is in direction d's queue; 0 between queries
+    uint32_t *fa, *fb;   // two frontiers of up to 2 n entries (vertex | direction << 31)
+    uint32_t *touched;   // labels set, up to 2 n vertices
     uint32_t nslots;
 };
 
-__device__ void dense_search(uint32_t root, uint32_t *dist, uint32_t *fst, uint32_t *fa,
-                             uint32_t *fb, uint32_t *touched, uint32_t *s_nt, uint32_t *s_nf,
-                             const uint32_t *off, const uint2 *adj, uint32_t n,
-                             uint32_t n_edges, uint32_t *err, uint32_t &stamp) {
-    const uint32_t tid = threadIdx.x;
-    if (tid == 0) {
-        dist[root] = 0;
-        touched[(*s_nt)++] = root;
-        fa[0] = root;
-        s_nf[0] = 1;
-    }
-    __syncthreads();
-    uint32_t *cur = fa, *nx = fb;
-    uint32_t c = 0;
-    while (true) {
-        const uint32_t nf = s_nf[c];
-        if (nf == 0) break;
-        ++stamp;
-        __syncthreads();
-        if (tid == 0) s_nf[c ^ 1] = 0;
-        __syncthreads();
-        for (uint32_t f = tid; f < nf; f += blockDim.x) {
-            const uint32_t x = cur[f];
-            if (x >= n) {
-                atomicOr(err, QERR_BOUND);
-                continue;
-            }
-            const uint32_t dx = dist[x];
-            const uint32_t jb = off[x], je = off[x + 1];
-            if (jb > je || je > n_edges) {
-                atomicOr(err, QERR_BOUND);
-                continue;
-            }
-            for (uint32_t j = jb; j < je; ++j) {
-                const uint2 e = adj[j];
-                const uint32_t nd = sat_add(dx, e.y);
-                if (nd == INF) continue;
-                if (e.x >= n) {
-                    atomicOr(err, QERR_BOUND);
-                    continue;
-                }
-                const uint32_t old = atomicMin(&dist[e.x], nd);
-                if (nd < old) {
-                    if (old == INF) touched[atomicAdd(s_nt, 1u)] = e.x;
-                    if (atomicExch(&fst[e.x], stamp) != stamp) nx[atomicAdd(&s_nf[c ^ 1], 1u)] = e.x;
-                }
-            }
-        }
-        __syncthreads();
-        uint32_t *t = cur;
-        cur = nx;
-        nx = t;
-        c ^= 1u;
-    }
-}
+constexpr int QD_THREADS = 1024;
+constexpr uint32_t QD_WORDS = 9;  // uint32 per vertex of a slot
+// Edges a level should expand: with fewer than the low mark the next level's
+// bucket doubles, with more than the high mark it halves.
+constexpr uint32_t QD_EDGES_LOW = 4096, QD_EDGES_HIGH = 32768;
 
-__global__ void __launch_bounds__(256) k_query_dense(QArgs a, QDense dn) {
+struct QDSmem {
+    // one tile of frontier entries: exclusive prefix of their out-degrees,
+    // first edge index, label, direction
+    uint32_t excl[QD_THREADS], beg[QD_THREADS], lab[QD_THREADS];
+    uint8_t dir[QD_THREADS];
+    uint32_t wtot[QD_THREADS / 32];
+    uint32_t cnt3[3], lmin3[3][2];  // queue sizes and least queued labels per level (mod 3)
+    uint32_t item, nt, mu, delta, edges;
+};
+
+// Both searches of a query at once, label-correcting, in levels like the
+// shared-table search's (block_search): a level expands the queued vertices
+// within `delta` of their direction's least queued label, keeps the others
+// and drops those whose label is not below the best meeting sum mu. Inside the
+// core, whose edges both directions hold, a search need not reach past the
+// middle of the path: a core vertex x is dropped when its label plus the other
+// direction's least queued label is not below mu. (A path through x shorter
+// than mu then has its remainder at labels the other direction has settled,
+// x among them, so x already holds both labels and mu counts their sum.
+// Vertices below the core are never dropped for this: only their own
+// direction climbs to the core.) Exhaustive searches (not PRUNE) expand
+// everything at once.
+//
+// Bound by the level chain's round trips to L2 (queue, label, offsets, edge,
+// label): the edges of a tile of 1024 entries are spread over all 1024 threads
+// by a block-wide scan, so that a hub's row costs no more than as many edges
+// of small rows, and the bucket width follows the work of the level before
+// (a fixed one is wrong by orders of magnitude from one graph to the next).
+// RMAT 2^15 (5,648 core vertices), 96 queries: 1.0 ms; a thread per
+// frontier vertex, both searches exhaustive and one after the other, after
+// two passes of overflowing table searches: 445 ms.
+template <bool PRUNE>
+__global__ void __launch_bounds__(QD_THREADS) k_query_dense(QArgs a, QDense dn) {
+    __shared__ QDSmem q;
+    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const size_t base = (size_t)blockIdx.x * a.n;
-    uint32_t *df = dn.df + base, *db = dn.db + base, *fst = dn.fst + base;
-    uint32_t *fa = dn.fa + base, *fb = dn.fb + base, *touched = dn.touched + 2 * base;
-    __shared__ uint32_t s_item, s_nt, s_nf[2], s_mu;
-    const uint32_t tid = threadIdx.x;
-    const uint32_t novf = a.work[a.ovf_cnt];
-    uint32_t stamp = 0;
+    uint32_t *df = dn.df + base, *db = dn.db + base, *queued = dn.queued + base;
+    uint32_t *const fra = dn.fa + 2 * base, *const frb = dn.fb + 2 * base;
+    uint32_t *touched = dn.touched + 2 * base;
+    const uint32_t nitems = a.dense_first ? (uint32_t)a.k : a.work[a.ovf_cnt];
+    QStat stat;
     while (true) {
         __syncthreads();
-        if (tid == 0) {
-            s_item = atomicAdd(&a.work[1], 1u);
-            s_nt = 0;
-            s_mu = INF;
-        }
+        if (tid == 0) q.item = atomicAdd(&a.work[1], 1u);
         __syncthreads();
-        if (s_item >= novf) break;
-        const uint32_t i = a.ovf[s_item];
-        const uint32_t rs = a.rank[a.src[i]], rt = a.rank[a.dst[i]];
+        if (q.item >= nitems) break;
+        const uint32_t i = a.dense_first ? q.item : a.ovf[q.item];
+        const uint32_t s = i < a.k ? a.src[i] : INF, t = i < a.k ? a.dst[i] : INF;
+        const uint32_t rs = s < a.n ? a.rank[s] : INF, rt = t < a.n ? a.rank[t] : INF;
         if (rs >= a.n || rt >= a.n) {
-            if (tid == 0) atomicOr(a.err, QERR_BOUND);
+            if (tid == 0) {
+                atomicOr(a.err, s >= a.n || t >= a.n ? QERR_RANGE : QERR_BOUND);
+                if (i < a.k) {
+                    a.out[i] = INF;
+                    if (a.settled) a.settled[i] = 0;
+                }
+            }
             continue;
         }
-        // forward labels live in df, backward in db; touched lists both
-        dense_search(rs, df, fst, fa, fb, touched, &s_nt, s_nf, a.up_off, a.up_adj, a.n, a.n_up,
-                     a.err, stamp);
-        __syncthreads();
-        const uint32_t nt_f = s_nt;
-        dense_search(rt, db, fst, fa, fb, touched, &s_nt, s_nf, a.dn_off, a.dn_adj, a.n, a.n_dn,
-                     a.err, stamp);
-        __syncthreads();
-        const uint32_t nt = s_nt;
-        // The touched list holds each vertex reached forward once (first nt_f
-        // entries), then each vertex reached backward once; every meeting
-        // vertex is in the forward part.
-        uint32_t mu = INF;
-        for (uint32_t p = tid; p < nt_f; p += blockDim.x) {
-            const uint32_t v = touched[p];
-            mu = min(mu, sat_add(df[v], db[v]));
+        if (tid == 0) {
+            df[rs] = 0;
+            db[rt] = 0;
+            queued[rs] = rs == rt ? 3u : 1u;
+            if (rs != rt) queued[rt] = 2u;
+            touched[0] = rs;
+            touched[1] = rt;
+            fra[0] = rs;
+            fra[1] = rt | 0x80000000u;
+            q.nt = 2;
+            q.mu = rs == rt ? 0u : INF;
+            q.cnt3[0] = 2;
+            q.cnt3[1] = 0;
+            q.lmin3[0][0] = q.lmin3[0][1] = 0;
+            q.lmin3[1][0] = q.lmin3[1][1] = INF;
+            q.delta = a.dense_delta;
+            q.edges = 0;
         }
-        atomicMin(&s_mu, mu);
+        for (uint32_t lvl = 0;; ++lvl) {
+            __syncthreads();
+            const uint32_t nfront = q.cnt3[lvl % 3];
+            const uint32_t mu0 = q.mu, minf = q.lmin3[lvl % 3][0], minb = q.lmin3[lvl % 3][1];
+            uint32_t delta = q.delta;
+            const uint32_t did = q.edges;
+            if (nfront == 0) break;
+            if (lvl >= (1u << 30)) {  // the least label grows every other level at the latest
+                if (tid == 0) atomicOr(a.err, QERR_BOUND);
+                break;
+            }
+            if (lvl && did < QD_EDGES_LOW) delta = min(2u * delta, 1u << 30);
+            else if (did > QD_EDGES_HIGH) delta = max(delta / 2u, 1u);
+            const uint32_t thrf = sat_add(minf, delta), thrb = sat_add(minb, delta);
+            __syncthreads();
+            if (tid == 0) {
+                q.cnt3[(lvl + 2) % 3] = 0;
+                q.lmin3[(lvl + 2) % 3][0] = q.lmin3[(lvl + 2) % 3][1] = INF;
+                q.delta = delta;
+                q.edges = 0;
+            }
+            const uint32_t *cur = lvl & 1u ? frb : fra;
+            uint32_t *nxt = lvl & 1u ? fra : frb;
+            uint32_t *ncnt = &q.cnt3[(lvl + 1) % 3];
+            uint32_t lmf = INF, lmb = INF;  // least labels this thread queues
+            for (uint32_t t0 = 0; t0 < nfront; t0 += QD_THREADS) {
+                const uint32_t fi = t0 + tid;
+                const uint32_t ent = fi < nfront ? __ldcg(cur + fi) : 0;
+                const uint32_t x = ent & 0x7FFFFFFFu, dir = ent >> 31;
+                bool ok = fi < nfront && x < a.n;
+                if (fi < nfront && !ok) atomicOr(a.err, QERR_BOUND);
+                uint32_t *dist = dir ? db : df;
+                uint32_t lab = ok ? __ldcg(dist + x) : INF;
+                bool keep = false;
+                if (PRUNE) {
+                    const bool drop = ok && (lab >= mu0 || (x >= a.core_first &&
+                                                            sat_add(lab, dir ? minf : minb) >= mu0));
+                    keep = ok && !drop && lab > (dir ? thrb : thrf);
+                    if (drop) {
+                        // a label lowered meanwhile is queued again
+                        atomicAnd(&queued[x], ~(1u << dir));
+                        const uint32_t now = __ldcg(dist + x);
+                        if (now < lab) {
+                            lab = now;
+                            if (!(atomicOr(&queued[x], 1u << dir) & (1u << dir))) keep = true;
+                        }
+                        ok = false;
+                    }
+                    const uint32_t m = __ballot_sync(FULL, keep);
+                    if (m) {
+                        uint32_t p = 0;
+                        const uint32_t leader = __ffs(m) - 1;
+                        if (lane == leader) p = atomicAdd(ncnt, (uint32_t)__popc(m));
+                        p = __shfl_sync(FULL, p, leader) + __popc(m & ((1u << lane) - 1u));
+                        if (keep) {
+                            if (p < 2u * a.n) nxt[p] = ent;
+                            else atomicOr(a.err, QERR_BOUND);
+                            if (dir) lmb = min(lmb, lab);
+                            else lmf = min(lmf, lab);
+                        }
+                    }
+                    if (keep) ok = false;
+                }
+                uint32_t b = 0, cnt = 0;
+                if (ok) {
+                    // out of the queue first, then its label: one lowered after
+                    // this read queues the vertex again
+                    atomicAnd(&queued[x], ~(1u << dir));
+                    lab = __ldcg(dist + x);
+                    const uint32_t *off = dir ? a.dn_off : a.up_off;
+                    b = off[x];
+                    const uint32_t e = off[x + 1];
+                    if (b <= e && e <= (dir ? a.n_dn : a.n_up)) cnt = e - b;
+                    else atomicOr(a.err, QERR_BOUND);
+                }
+                stat.exp += cnt ? 1u : 0u;
+                const uint32_t incl = warp_incl_scan(cnt);
+                if (lane == 31) q.wtot[warp] = incl;
+                q.beg[tid] = b;
+                q.lab[tid] = lab;
+                q.dir[tid] = (uint8_t)dir;
+                __syncthreads();
+                const uint32_t wt = q.wtot[lane];
+                const uint32_t wincl = warp_incl_scan(wt);
+                const uint32_t total = __shfl_sync(FULL, wincl, 31);
+                q.excl[tid] = __shfl_sync(FULL, wincl - wt, warp) + incl - cnt;
+                if (tid == 0) q.edges += total;
+                __syncthreads();
+                for (uint32_t e0 = tid; e0 < total; e0 += QD_THREADS) {
+                    // owner entry: the largest k with excl[k] <= e0
+                    uint32_t k = 0;
+#pragma unroll
+                    for (uint32_t step = QD_THREADS / 2; step > 0; step >>= 1)
+                        if (q.excl[k + step] <= e0) k += step;
+                    ++stat.edges;
+                    const uint32_t edir = q.dir[k];
+                    const uint2 e = (edir ? a.dn_adj : a.up_adj)[q.beg[k] + (e0 - q.excl[k])];
+                    const uint32_t nd = sat_add(q.lab[k], e.y);
+                    if (e.x >= a.n) {
+                        atomicOr(a.err, QERR_BOUND);
+                        continue;
+                    }
+                    if (nd == INF) continue;
+                    if (PRUNE && nd >= *(volatile uint32_t *)&q.mu) continue;
+                    uint32_t *ed = edir ? db : df;
+                    if (nd >= __ldcg(ed + e.x)) continue;
+                    const uint32_t old = atomicMin(&ed[e.x], nd);
+                    if (nd >= old) continue;
+                    if (old == INF) {
+                        const uint32_t p = atomicAdd(&q.nt, 1u);
+                        if (p < 2u * a.n) touched[p] = e.x;
+                        else atomicOr(a.err, QERR_BOUND);
+                    }
+                    if (edir) lmb = min(lmb, nd);
+                    else lmf = min(lmf, nd);
+                    if (PRUNE) {
+                        const uint32_t other = __ldcg((edir ? df : db) + e.x);
+                        if (other != INF) atomicMin(&q.mu, sat_add(nd, other));
+                    }
+                    if (!(atomicOr(&queued[e.x], 1u << edir) & (1u << edir))) {
+                        const uint32_t p = atomicAdd(ncnt, 1u);
+                        if (p < 2u * a.n) nxt[p] = e.x | (edir << 31);
+                        else atomicOr(a.err, QERR_BOUND);
+                    }
+                }
+                __syncthreads();
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                lmf = min(lmf, __shfl_xor_sync(FULL, lmf, o));
+                lmb = min(lmb, __shfl_xor_sync(FULL, lmb, o));
+            }
+            if (lane == 0) {
+                if (lmf != INF) atomicMin(&q.lmin3[(lvl + 1) % 3][0], lmf);
+                if (lmb != INF) atomicMin(&q.lmin3[(lvl + 1) % 3][1], lmb);
+            }
+        }
+        __syncthreads();
+        // the answer: the least meeting sum over the vertices reached
+        const uint32_t nt = min(q.nt, 2u * a.n);
+        if (tid == 0) q.mu = INF;
+        __syncthreads();
+        uint32_t mu = INF;
+        for (uint32_t p = tid; p < nt; p += QD_THREADS) {
+            const uint32_t v = __ldcg(touched + p);
+            mu = min(mu, sat_add(__ldcg(df + v), __ldcg(db + v)));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mu = min(mu, __shfl_xor_sync(FULL, mu, o));
+        if (lane == 0 && mu != INF) atomicMin(&q.mu, mu);
         __syncthreads();
         if (tid == 0) {
-            a.out[i] = s_mu;
+            a.out[i] = q.mu;
             if (a.settled) a.settled[i] = nt;
         }
-        __syncthreads();
-        for (uint32_t p = tid; p < nt; p += blockDim.x) {
-            const uint32_t v = touched[p];
+        for (uint32_t p = tid; p < nt; p += QD_THREADS) {
+            const uint32_t v = __ldcg(touched + p);
             df[v] = INF;
             db[v] = INF;
-            fst[v] = 0;
+            queued[v] = 0;
         }
     }
+    qb_flush_stat(stat, a.stats);
 }
 
 // Resident blocks per SM of each block-kernel configuration
@@ -288,13 +430,14 @@ void query_init(ch_s *h) {
     h->qwork.alloc(8);
     h->q_ovf_cap = Q_CHUNK;
     h->q_ovf_list.alloc(2 * Q_CHUNK);  // overflow lists of the two block-kernel passes
-    // per slot: df, db, fst, two frontiers (n each) and the touched list
-    // of both directions (2n)
-    const uint64_t per_slot = (uint64_t)std::max<uint32_t>(n, 1) * 7 * 4;
-    h->q_slots = (uint32_t)std::max<uint64_t>(2, std::min<uint64_t>(64, (1024ull << 20) / per_slot));
-    h->q_dense.alloc((size_t)h->q_slots * std::max<uint32_t>(n, 1) * 7);
+    // as many slots as the chip runs blocks of the dense kernel at once (two
+    // an SM), within 1 GiB
+    const uint64_t per_slot = (uint64_t)std::max<uint32_t>(n, 1) * QD_WORDS * 4;
+    h->q_slots = (uint32_t)std::max<uint64_t>(
+        2, std::min<uint64_t>(2 * (uint64_t)device_sm_count(), (1024ull << 20) / per_slot));
     const size_t sn = (size_t)h->q_slots * std::max<uint32_t>(n, 1);
-    // df, db: INF; fst: 0; the rest need no initial value
+    h->q_dense.alloc(sn * QD_WORDS);
+    // df, db: INF; queue bits: 0; the rest need no initial value
     CH_CUDA_TRY(cudaMemset(h->q_dense.ptr, 0xFF, sn * 2 * 4));
     CH_CUDA_TRY(cudaMemset(h->q_dense.ptr + 2 * sn, 0, sn * 4));
     h->q_stats.alloc(2);
@@ -320,47 +463,85 @@ void query_init(ch_s *h) {
     CH_CUDA_TRY(cudaDeviceSynchronize());
 }
 
-void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
-                 uint32_t *dist_out, uint32_t *settled_out, cudaStream_t st) {
-    if (k == 0) return;
+namespace {
+
+// The label arrays of the dense kernel's slots.
+QDense dense_slots(const ch_s *h) {
     const size_t sn = (size_t)h->q_slots * std::max<uint32_t>(h->n, 1);
     QDense dn;
     dn.df = h->q_dense.ptr;
     dn.db = dn.df + sn;
-    dn.fst = dn.df + 2 * sn;
+    dn.queued = dn.df + 2 * sn;
     dn.fa = dn.df + 3 * sn;
-    dn.fb = dn.df + 4 * sn;
-    dn.touched = dn.df + 5 * sn;  // 2 * sn entries
+    dn.fb = dn.df + 5 * sn;
+    dn.touched = dn.df + 7 * sn;
     dn.nslots = h->q_slots;
+    return dn;
+}
+
+// Searches of a core larger than this reach more vertices than a table of
+// 2^12 slots takes, so their queries go to the dense kernel at once (without
+// a core table, which keeps the searches out of the core). Half the table:
+// the searches below the core need room too. 96 queries of RMAT 2^15 (core
+// 5,648): 320 ms of the 445 were the two passes that overflowed.
+constexpr uint64_t DENSE_FIRST_CORE = 2048;
+
+// What every kernel of a batch needs of the hierarchy.
+QArgs hierarchy_args(const ch_s *h) {
+    QArgs a;
+    a.n = h->n;
+    a.n_up = (uint32_t)h->n_up;
+    a.n_dn = (uint32_t)h->n_down;
+    a.rank = h->rank.ptr;
+    a.up_off = h->up_off.ptr;
+    a.dn_off = h->dn_off.ptr;
+    a.up_adj = h->up_adj.ptr;
+    a.dn_adj = h->dn_adj.ptr;
+    a.err = h->qerr.ptr;
+    a.stats = h->q_stats.ptr;
+    a.core_tab = h->core_n ? h->core_tab.ptr : nullptr;
+    a.core_lo = h->core_lo;
+    a.core_n = h->core_n;
+    a.core_first = (uint32_t)(h->n - h->core_size);
+    a.dense_delta = std::max<uint32_t>(1, h->q_wscale / 8);
+    a.dense_first = !h->core_n && h->core_size > DENSE_FIRST_CORE;
+    a.delta = h->q_delta ? h->q_delta : INF;
+    return a;
+}
+
+// The dense kernel over a batch's overflowed queries (or all of them).
+void launch_query_dense(const ch_s *h, const QArgs &a, bool prune, uint64_t k, cudaStream_t st) {
+    const QDense dn = dense_slots(h);
+    const unsigned blocks = (unsigned)std::min<uint64_t>(dn.nslots, k);
+    if (prune) k_query_dense<true><<<blocks, QD_THREADS, 0, st>>>(a, dn);
+    else k_query_dense<false><<<blocks, QD_THREADS, 0, st>>>(a, dn);
+    CH_CHECK_LAUNCH();
+}
+
+}  // namespace
+
+void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
+                 uint32_t *dist_out, uint32_t *settled_out, cudaStream_t st) {
+    if (k == 0) return;
     for (uint64_t c0 = 0; c0 < k; c0 += Q_CHUNK) {
         const uint64_t kc = std::min<uint64_t>(Q_CHUNK, k - c0);
-        QArgs a;
-        a.n = h->n;
-        a.n_up = (uint32_t)h->n_up;
-        a.n_dn = (uint32_t)h->n_down;
-        a.rank = h->rank.ptr;
-        a.up_off = h->up_off.ptr;
-        a.dn_off = h->dn_off.ptr;
-        a.up_adj = h->up_adj.ptr;
-        a.dn_adj = h->dn_adj.ptr;
+        QArgs a = hierarchy_args(h);
         a.src = src + c0;
         a.dst = dst + c0;
         a.out = dist_out + c0;
         a.settled = settled_out ? settled_out + c0 : nullptr;
         a.k = kc;
         a.work = h->qwork.ptr;
-        a.err = h->qerr.ptr;
-        a.stats = h->q_stats.ptr;
         a.in_list = nullptr;
         a.in_cnt = 0;
-        a.core_tab = h->core_n ? h->core_tab.ptr : nullptr;
-        a.core_lo = h->core_lo;
-        a.core_n = h->core_n;
-        a.delta = h->q_delta ? h->q_delta : INF;
         CH_CUDA_TRY(cudaMemsetAsync(h->qwork.ptr, 0, 8 * sizeof(uint32_t), st));
         // Pruned searches unless the caller asked for search-space sizes,
         // which are defined by the exhaustive upward searches.
         const bool prune = settled_out == nullptr;
+        if (a.dense_first) {
+            launch_query_dense(h, a, prune, kc, st);
+            continue;
+        }
         if (h->q_small_first) {
             // pass 1 on small tables (twice the resident queries); the
             // queries that overflow them are redone on the large tables
@@ -376,8 +557,7 @@ void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
         a.ovf = h->q_ovf_list.ptr;
         a.ovf_cnt = 2;
         launch_query_block(h, a, prune, false, kc, st);
-        k_query_dense<<<h->q_slots, 256, 0, st>>>(a, dn);
-        CH_CHECK_LAUNCH();
+        launch_query_dense(h, a, prune, kc, st);
     }
 }
 
@@ -640,24 +820,7 @@ void query_batch_static(ch_s *h, const uint32_t *src, const uint32_t *dst, uint6
     if (dev != h->device)
         throw Error{CH_EINVAL, "the current device is not the hierarchy's device"};
     uint32_t *scratch = static_scratch();
-    const size_t sn = (size_t)h->q_slots * std::max<uint32_t>(h->n, 1);
-    QDense dn;
-    dn.df = h->q_dense.ptr;
-    dn.db = dn.df + sn;
-    dn.fst = dn.df + 2 * sn;
-    dn.fa = dn.df + 3 * sn;
-    dn.fb = dn.df + 4 * sn;
-    dn.touched = dn.df + 5 * sn;
-    dn.nslots = h->q_slots;
-    QArgs a;
-    a.n = h->n;
-    a.n_up = (uint32_t)h->n_up;
-    a.n_dn = (uint32_t)h->n_down;
-    a.rank = h->rank.ptr;
-    a.up_off = h->up_off.ptr;
-    a.dn_off = h->dn_off.ptr;
-    a.up_adj = h->up_adj.ptr;
-    a.dn_adj = h->dn_adj.ptr;
+    QArgs a = hierarchy_args(h);
     a.src = src;
     a.dst = dst;
     a.out = dist_out;
@@ -669,18 +832,11 @@ void query_batch_static(ch_s *h, const uint32_t *src, const uint32_t *dst, uint6
     a.ctr = 0;
     a.ovf = scratch + kStaticScratchHead;
     a.ovf_cnt = 2;
-    a.err = h->qerr.ptr;
-    a.stats = h->q_stats.ptr;
-    a.core_tab = h->core_n ? h->core_tab.ptr : nullptr;
-    a.core_lo = h->core_lo;
-    a.core_n = h->core_n;
-    a.delta = h->q_delta ? h->q_delta : INF;
     // the counters keep the previous call's values: clear them
     CH_CUDA_TRY(cudaMemsetAsync(scratch, 0, kStaticScratchHead * sizeof(uint32_t), st));
     // one block-kernel pass (large tables): the scratch holds one list
-    launch_query_block(h, a, true, false, k, st);
-    k_query_dense<<<h->q_slots, 256, 0, st>>>(a, dn);
-    CH_CHECK_LAUNCH();
+    if (!a.dense_first) launch_query_block(h, a, true, false, k, st);
+    launch_query_dense(h, a, true, k, st);
 }
 
 }  // namespace gbch

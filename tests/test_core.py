@@ -210,3 +210,31 @@ def test_core_table_byte_limit():
     assert np.array_equal(gch.query(s, t), O.dijkstra_pairs(g, s, t))  # no table: the full search
     gch.core_table(max_bytes=4 * core * core)
     assert np.array_equal(gch.query(s, t), O.dijkstra_pairs(g, s, t))
+
+
+# A core above half a shared table's slots: its queries go to the per-vertex
+# label arrays at once. With cmax = 0 nearly every vertex stays in the core.
+@pytest.mark.parametrize("n,seed", [(2300, 102), (6001, 103)])
+def test_queries_of_a_large_core(n, seed):
+    torch = pytest.importorskip("torch")
+    g = I.geometric_knn_graph(n, seed=seed)
+    och = O.build_ch(g, 5, cmax=0)
+    gch = _ch().CH.build(g, hop_limit=5, max_candidates_per_vertex=0)
+    assert gch.stats()["core_vertices"] > 2048
+    s, t = I.random_pairs(g.n, 700, seed=seed)
+    t[:20] = s[:20]  # the source itself
+    d = assert_same_queries(gch, och, s, t)  # exhaustive searches, sizes included
+    assert np.array_equal(d, O.dijkstra_pairs(g, s, t))
+    assert np.array_equal(gch.query(s, t), d)
+    ds, dt = (torch.from_numpy(x.view(np.int32)).cuda() for x in (s, t))
+    assert np.array_equal(gch.query_one_to_many(int(s[0]), dt).cpu().numpy().view(np.uint32),
+                          O.dijkstra_pairs(g, np.full_like(t, s[0]), t))
+    # an id out of range is reported, its answer INF, the others unharmed
+    ds[3] = g.n
+    got = gch.query(ds, dt).cpu().numpy().view(np.uint32)
+    with pytest.raises(_ch().CHError) as ei:
+        gch.query_status()
+    assert ei.value.code == _ch().CH_EINVAL
+    want = d.copy()
+    want[3] = 0xFFFFFFFF
+    assert np.array_equal(got, want)
