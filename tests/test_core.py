@@ -238,3 +238,15 @@ def test_queries_of_a_large_core(n, seed):
     want = d.copy()
     want[3] = 0xFFFFFFFF
     assert np.array_equal(got, want)
+
+
+# Labels in shared memory up to 51,200 core vertices, in the table's row above.
+@pytest.mark.parametrize("n,seed", [(4000, 104), (52_500, 105)])
+def test_core_table_label_placements(n, seed):
+    g = I.geometric_knn_graph(n, seed=seed)
+    gch = _ch().CH.build(g, hop_limit=5, max_candidates_per_vertex=0)
+    core = gch.stats()["core_vertices"]
+    assert core > (51_200 if n > 50_000 else 2048)
+    gch.core_table()
+    s, t = I.random_pairs(g.n, 300, seed=seed)
+    assert np.array_equal(gch.query(s, t), O.dijkstra_pairs(g, s, t))
