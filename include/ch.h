@@ -234,7 +234,13 @@ int ch_build(const ch_graph_t *g, const ch_params_t *params, ch_t **out);
  * `stream` (a cudaStream_t, NULL = legacy stream) and the call returns
  * without waiting. Ids >= n give CH_EINVAL for the whole batch (checked on
  * the device; the status is returned by the next synchronising call on the
- * handle, or by ch_query_status). k = 0 is a no-op. */
+ * handle, or by ch_query_status). k = 0 is a no-op.
+ * A batch of at least 2^14 and 60 sqrt(n) queries (without settled_out, on a
+ * hierarchy without a core and of at most about 4M vertices) is answered
+ * through hub labels computed by the call for the vertices the batch climbs
+ * through; the first such batch of a handle allocates their memory (about 6 KB
+ * a vertex, kept until ch_free; without that memory, or in a stream capture
+ * before it exists, the batch is searched query by query). Same answers. */
 int ch_query_batch(ch_t *ch, const uint32_t *src, const uint32_t *dst, uint64_t k,
                    uint32_t *dist_out, uint32_t *settled_out, void *stream);
 
@@ -386,7 +392,8 @@ int ch_build_autotune(const ch_graph_t *graph, const ch_params_t *params,
 /* Work of the query searches since the previous call (then cleared), summed
  * over the handle's batches: out[0] = queued entries expanded (a stalled
  * entry counts: its stall test read it), out[1] = adjacency entries scanned,
- * the stall tests' included. Waits for `stream`. */
+ * the stall tests' included. A batch answered through hub labels counts its
+ * labels and the label and stall-test entries read. Waits for `stream`. */
 int ch_query_work(ch_t *ch, void *stream, uint64_t out[2]);
 
 /* ---- Query batches as CUDA graphs ----

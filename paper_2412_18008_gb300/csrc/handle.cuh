@@ -72,6 +72,14 @@ struct ch_s {
     uint64_t q_ovf_cap = 0;
     gbch::DevBuf<uint32_t> q_src_fill;  // repeated source of one-to-many queries
 
+    // Label memory of large batches (hublabel.cu), made by the first of them
+    gbch::DevBuf<uint2> hl_arena;
+    gbch::DevBuf<uint32_t> hl_label;  // arena position, then size, of each label [2][2 n]
+    gbch::DevBuf<uint8_t> hl_mark;
+    gbch::DevBuf<uint32_t> hl_list;
+    gbch::DevBuf<unsigned long long> hl_cursor;
+    bool hl_off = false;  // no memory for labels, or a hierarchy they cannot serve
+
     // One-to-all scratch: interleaved labels of a batch of sources, level
     // boundaries, the core pass's change flag.
     gbch::DevBuf<uint32_t> phast_d;
@@ -90,9 +98,22 @@ namespace gbch {
 // Build a hierarchy into `h` (h->n etc. are set by the callee).
 void build_hierarchy(ch_s *h, const ch_graph_t *g, const ch_params_t *p);
 
-// Enqueue a query batch on `st` (device pointers).
+// Enqueue a query batch on `st` (device pointers); with searches_only, large
+// batches too are answered by one search a query.
 void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
-                 uint32_t *dist_out, uint32_t *settled_out, cudaStream_t st);
+                 uint32_t *dist_out, uint32_t *settled_out, cudaStream_t st, bool searches_only = false);
+
+// Large batches by hub labels (hublabel.cu). prepare: allocates their memory;
+// whether a batch of k queries would use them. batch: answers the batch on
+// `st`, appending queries it could not answer to ovf (count in *ovf_cnt);
+// false, with nothing done, when the batch is for the searches.
+bool query_labels_prepare(ch_s *h, uint64_t k);
+bool query_batch_labels(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k, uint32_t *dist_out,
+                        uint32_t *ovf, uint32_t *ovf_cnt, cudaStream_t st);
+
+// Level boundaries in rank order: level l holds ranks [lv[l], lv[l + 1]), the
+// last entry pair the core. False if the levels do not add up to n vertices.
+bool rank_levels(const ch_s *h, std::vector<uint32_t> &lv);
 
 // Prepare query scratch after a build.
 void query_init(ch_s *h);

@@ -170,20 +170,25 @@ __global__ void k_phast_out(const uint32_t *D, const uint32_t *rank, uint32_t n,
 
 }  // namespace
 
+bool rank_levels(const ch_s *h, std::vector<uint32_t> &lv) {
+    const size_t L = h->round_stats.size();
+    lv.resize(L + 2);
+    uint64_t acc = 0;
+    for (size_t l = 0; l < L; ++l) {
+        lv[l] = (uint32_t)std::min<uint64_t>(acc, h->n);
+        acc += h->round_stats[l][2];  // |V_F| of round l
+    }
+    lv[L] = (uint32_t)std::min<uint64_t>(acc, h->n);
+    lv[L + 1] = h->n;
+    return acc + h->core_size == h->n;
+}
+
 void one_to_all(ch_s *h, const uint32_t *src, uint64_t k, uint32_t *dist_out, cudaStream_t st) {
     if (k == 0 || h->n == 0) return;
     const uint32_t n = h->n;
-    // Level boundaries in rank order: round r's selected count, then the core.
     const size_t L = h->round_stats.size();
-    std::vector<uint32_t> lv(L + 2);
-    uint64_t acc = 0;
-    for (size_t l = 0; l < L; ++l) {
-        lv[l] = (uint32_t)std::min<uint64_t>(acc, n);
-        acc += h->round_stats[l][2];  // |V_F| of round l
-    }
-    lv[L] = (uint32_t)std::min<uint64_t>(acc, n);
-    lv[L + 1] = n;
-    if (acc + h->core_size != n) throw Error{CH_EINVAL, "the hierarchy's level sizes do not add up to n"};
+    std::vector<uint32_t> lv;
+    if (!rank_levels(h, lv)) throw Error{CH_EINVAL, "the hierarchy's level sizes do not add up to n"};
     // The tail: the longest run of small levels right below the core.
     size_t tail = L;
     while (tail > 0 && lv[tail] - lv[tail - 1] <= TAIL_MAX) --tail;

@@ -521,7 +521,7 @@ void launch_query_dense(const ch_s *h, const QArgs &a, bool prune, uint64_t k, c
 }  // namespace
 
 void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
-                 uint32_t *dist_out, uint32_t *settled_out, cudaStream_t st) {
+                 uint32_t *dist_out, uint32_t *settled_out, cudaStream_t st, bool searches_only) {
     if (k == 0) return;
     for (uint64_t c0 = 0; c0 < k; c0 += Q_CHUNK) {
         const uint64_t kc = std::min<uint64_t>(Q_CHUNK, k - c0);
@@ -542,7 +542,12 @@ void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
             launch_query_dense(h, a, prune, kc, st);
             continue;
         }
-        if (h->q_small_first) {
+        if (prune && !searches_only &&
+            query_batch_labels(h, a.src, a.dst, kc, a.out, h->q_ovf_list.ptr + Q_CHUNK, h->qwork.ptr + 4, st)) {
+            // the queries that the labels could not answer, by searches
+            a.in_list = h->q_ovf_list.ptr + Q_CHUNK;
+            a.in_cnt = 4;
+        } else if (h->q_small_first) {
             // pass 1 on small tables (twice the resident queries); the
             // queries that overflow them are redone on the large tables
             a.ctr = 0;
@@ -627,9 +632,9 @@ void query_autotune(ch_s *h, uint64_t sample, uint32_t seed, cudaStream_t st, ch
     try {
         for (int i = 0; i < CH_QUERY_AUTOTUNE_CONFIGS; ++i) {
             apply(i);
-            query_batch(h, s, t, sample, out, nullptr, st);  // warm-up
+            query_batch(h, s, t, sample, out, nullptr, st, true);  // warm-up
             CH_CUDA_TRY(cudaEventRecord(e0, st));
-            query_batch(h, s, t, sample, out, nullptr, st);
+            query_batch(h, s, t, sample, out, nullptr, st, true);
             CH_CUDA_TRY(cudaEventRecord(e1, st));
             CH_CUDA_TRY(cudaEventSynchronize(e1));
             float ms = 0;
@@ -678,9 +683,9 @@ double query_time_sample(ch_s *h, uint64_t sample, uint32_t seed, cudaStream_t s
     float ms = 0;
     cudaError_t e = cudaSuccess;
     try {
-        query_batch(h, s, t, sample, out, nullptr, st);  // warm-up
+        query_batch(h, s, t, sample, out, nullptr, st, true);  // warm-up
         CH_CUDA_TRY(cudaEventRecord(e0, st));
-        query_batch(h, s, t, sample, out, nullptr, st);
+        query_batch(h, s, t, sample, out, nullptr, st, true);
         CH_CUDA_TRY(cudaEventRecord(e1, st));
         CH_CUDA_TRY(cudaEventSynchronize(e1));
         e = cudaEventElapsedTime(&ms, e0, e1);
@@ -717,6 +722,7 @@ namespace gbch {
 
 ch_query_graph_s *query_graph_create(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
                                      uint32_t *dist_out) {
+    query_labels_prepare(h, std::min<uint64_t>(k, Q_CHUNK));  // a capture must not allocate
     cudaStream_t st = nullptr;
     CH_CUDA_TRY(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
     cudaGraph_t graph = nullptr;
