@@ -103,6 +103,11 @@ void build_hierarchy(ch_s *h, const ch_graph_t *g, const ch_params_t *p);
 void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
                  uint32_t *dist_out, uint32_t *settled_out, cudaStream_t st, bool searches_only = false);
 
+// Small batches by one block of 1024 threads a query, in one launch (src null:
+// every source is one_src). False, with nothing done, for other batches.
+bool query_batch_small(ch_s *h, const uint32_t *src, uint32_t one_src, const uint32_t *dst, uint64_t k,
+                       uint32_t *dist_out, cudaStream_t st);
+
 // Large batches by hub labels (hublabel.cu). prepare: allocates their memory;
 // whether a batch of k queries would use them. batch: answers the batch on
 // `st`, appending queries it could not answer to ovf (count in *ovf_cnt);

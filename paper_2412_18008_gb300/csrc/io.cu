@@ -188,7 +188,7 @@ ch_s *load_hierarchy(const char *path) {
 
 void query_one_to_many(ch_s *h, uint32_t s, const uint32_t *dst, uint64_t k, uint32_t *dist_out,
                        cudaStream_t st) {
-    if (k == 0) return;
+    if (k == 0 || query_batch_small(h, nullptr, s, dst, k, dist_out, st)) return;
     if (h->q_src_fill.count < k) h->q_src_fill.alloc(k);
     k_fill<<<grid_for(k, 256, device_sm_count() * 4), 256, 0, st>>>(h->q_src_fill.ptr, k, s);
     CH_CHECK_LAUNCH();

@@ -52,7 +52,8 @@ struct QArgs {
     const uint32_t *rank;
     const uint32_t *up_off, *dn_off;
     const uint2 *up_adj, *dn_adj;
-    const uint32_t *src, *dst;
+    const uint32_t *src, *dst;  // src null (small batches): every source is one_src
+    uint32_t one_src;
     uint32_t *out, *settled;
     uint64_t k;
     // Work items and counters. A block kernel takes items from work[ctr]:
@@ -62,7 +63,7 @@ struct QArgs {
     // dense_first, all queries) from work[1].
     uint32_t *work;
     const uint32_t *in_list;
-    uint32_t in_cnt, ctr, ovf_cnt;
+    uint32_t in_cnt, ctr, ovf_cnt, ticket;  // (ticket: the dense kernel's finished blocks, the last counter)
     uint32_t *ovf;
     uint32_t *err;
     unsigned long long *stats;  // [0] expansions, [1] edges scanned (or null)
@@ -463,9 +464,10 @@ __device__ __forceinline__ void qb_clear(QBSmem<TB> &q) {
 // overflowed the table or the frontier (the caller redoes the query
 // elsewhere); otherwise mu and cnt hold, in every thread, the least meeting
 // sum and the number of labels set. Every thread of the block must call it.
-template <bool PRUNE, bool WARP, int TB, bool STALL = false, bool DELTA = false>
-__device__ bool block_query(QBSmem<TB> &q, const QArgs &a, uint32_t rs, uint32_t rt, uint32_t &mu_out,
-                            uint32_t &cnt_out, QStat &stat) {
+// `search` runs the levels (block_search's contract).
+template <int TB, class S>
+__device__ bool block_query_by(QBSmem<TB> &q, const QArgs &a, uint32_t rs, uint32_t rt, uint32_t &mu_out,
+                               uint32_t &cnt_out, S &&search) {
     const uint32_t tid = threadIdx.x;
     __syncthreads();
     if (tid == 0) {
@@ -481,12 +483,10 @@ __device__ bool block_query(QBSmem<TB> &q, const QArgs &a, uint32_t rs, uint32_t
         q.cnt3[0] = 2;
         q.cnt3[1] = 0;
         q.cnt3[2] = 0;
-        if (DELTA) {
-            q.lmin3[0][0] = q.lmin3[0][1] = 0;  // the two roots
-            q.lmin3[1][0] = q.lmin3[1][1] = INF;
-        }
+        q.lmin3[0][0] = q.lmin3[0][1] = 0;  // the two roots
+        q.lmin3[1][0] = q.lmin3[1][1] = INF;
     }
-    bool ok = block_search<PRUNE, WARP, TB, STALL, DELTA>(q, a, stat);
+    bool ok = search();
     // q.mu only steered pruning; the answer is the least meeting sum.
     __syncthreads();
     if (tid == 0) {
@@ -550,6 +550,13 @@ __device__ bool block_query(QBSmem<TB> &q, const QArgs &a, uint32_t rs, uint32_t
     mu_out = q.mu;
     cnt_out = q.cnt;
     return ok;
+}
+
+template <bool PRUNE, bool WARP, int TB, bool STALL = false, bool DELTA = false>
+__device__ bool block_query(QBSmem<TB> &q, const QArgs &a, uint32_t rs, uint32_t rt, uint32_t &mu_out,
+                            uint32_t &cnt_out, QStat &stat) {
+    return block_query_by(q, a, rs, rt, mu_out, cnt_out,
+                          [&] { return block_search<PRUNE, WARP, TB, STALL, DELTA>(q, a, stat); });
 }
 
 // Adds the block's counters to stats[0] (expansions) and stats[1] (edges).

@@ -27,6 +27,9 @@ namespace gbch {
 namespace {
 
 constexpr uint64_t Q_CHUNK = 1u << 22;  // queries per launch pair
+// Counters of a batch: zero between batches (its last kernel, the dense one,
+// clears them), the last one counts that kernel's finished blocks.
+constexpr uint32_t QWORK = 8;
 
 // (The stalling variants are held to six resident blocks per SM, about 40
 // registers a thread, so that six 2^11-slot blocks fit an SM.)
@@ -119,6 +122,8 @@ struct QDSmem {
 // direction climbs to the core.) Exhaustive searches (not PRUNE) expand
 // everything at once.
 //
+// mu_out and cnt_out are, in every thread, the answer and the labels set.
+//
 // Bound by the level chain's round trips to L2 (queue, label, offsets, edge,
 // label): the edges of a tile of 1024 entries are spread over all 1024 threads
 // by a block-wide scan, so that a hub's row costs no more than as many edges
@@ -128,212 +133,354 @@ struct QDSmem {
 // frontier vertex, both searches exhaustive and one after the other, after
 // two passes of overflowing table searches: 445 ms.
 template <bool PRUNE>
-__global__ void __launch_bounds__(QD_THREADS) k_query_dense(QArgs a, QDense dn) {
-    __shared__ QDSmem q;
+__device__ void dense_query(QDSmem &q, const QArgs &a, const QDense &dn, uint32_t rs, uint32_t rt, uint32_t &mu_out,
+                            uint32_t &cnt_out, QStat &stat) {
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const size_t base = (size_t)blockIdx.x * a.n;
     uint32_t *df = dn.df + base, *db = dn.db + base, *queued = dn.queued + base;
     uint32_t *const fra = dn.fa + 2 * base, *const frb = dn.fb + 2 * base;
     uint32_t *touched = dn.touched + 2 * base;
+    __syncthreads();
+    if (tid == 0) {
+        df[rs] = 0;
+        db[rt] = 0;
+        queued[rs] = rs == rt ? 3u : 1u;
+        if (rs != rt) queued[rt] = 2u;
+        touched[0] = rs;
+        touched[1] = rt;
+        fra[0] = rs;
+        fra[1] = rt | 0x80000000u;
+        q.nt = 2;
+        q.mu = rs == rt ? 0u : INF;
+        q.cnt3[0] = 2;
+        q.cnt3[1] = 0;
+        q.lmin3[0][0] = q.lmin3[0][1] = 0;
+        q.lmin3[1][0] = q.lmin3[1][1] = INF;
+        q.delta = a.dense_delta;
+        q.edges = 0;
+    }
+    for (uint32_t lvl = 0;; ++lvl) {
+        __syncthreads();
+        const uint32_t nfront = q.cnt3[lvl % 3];
+        const uint32_t mu0 = q.mu, minf = q.lmin3[lvl % 3][0], minb = q.lmin3[lvl % 3][1];
+        uint32_t delta = q.delta;
+        const uint32_t did = q.edges;
+        if (nfront == 0) break;
+        if (lvl >= (1u << 30)) {  // the least label grows every other level at the latest
+            if (tid == 0) atomicOr(a.err, QERR_BOUND);
+            break;
+        }
+        if (lvl && did < QD_EDGES_LOW) delta = min(2u * delta, 1u << 30);
+        else if (did > QD_EDGES_HIGH) delta = max(delta / 2u, 1u);
+        const uint32_t thrf = sat_add(minf, delta), thrb = sat_add(minb, delta);
+        __syncthreads();
+        if (tid == 0) {
+            q.cnt3[(lvl + 2) % 3] = 0;
+            q.lmin3[(lvl + 2) % 3][0] = q.lmin3[(lvl + 2) % 3][1] = INF;
+            q.delta = delta;
+            q.edges = 0;
+        }
+        const uint32_t *cur = lvl & 1u ? frb : fra;
+        uint32_t *nxt = lvl & 1u ? fra : frb;
+        uint32_t *ncnt = &q.cnt3[(lvl + 1) % 3];
+        uint32_t lmf = INF, lmb = INF;  // least labels this thread queues
+        for (uint32_t t0 = 0; t0 < nfront; t0 += QD_THREADS) {
+            const uint32_t fi = t0 + tid;
+            const uint32_t ent = fi < nfront ? __ldcg(cur + fi) : 0;
+            const uint32_t x = ent & 0x7FFFFFFFu, dir = ent >> 31;
+            bool ok = fi < nfront && x < a.n;
+            if (fi < nfront && !ok) atomicOr(a.err, QERR_BOUND);
+            uint32_t *dist = dir ? db : df;
+            uint32_t lab = ok ? __ldcg(dist + x) : INF;
+            bool keep = false;
+            if (PRUNE) {
+                const bool drop = ok && (lab >= mu0 || (x >= a.core_first &&
+                                                        sat_add(lab, dir ? minf : minb) >= mu0));
+                keep = ok && !drop && lab > (dir ? thrb : thrf);
+                if (drop) {
+                    // a label lowered meanwhile is queued again
+                    atomicAnd(&queued[x], ~(1u << dir));
+                    const uint32_t now = __ldcg(dist + x);
+                    if (now < lab) {
+                        lab = now;
+                        if (!(atomicOr(&queued[x], 1u << dir) & (1u << dir))) keep = true;
+                    }
+                    ok = false;
+                }
+                const uint32_t m = __ballot_sync(FULL, keep);
+                if (m) {
+                    uint32_t p = 0;
+                    const uint32_t leader = __ffs(m) - 1;
+                    if (lane == leader) p = atomicAdd(ncnt, (uint32_t)__popc(m));
+                    p = __shfl_sync(FULL, p, leader) + __popc(m & ((1u << lane) - 1u));
+                    if (keep) {
+                        if (p < 2u * a.n) nxt[p] = ent;
+                        else atomicOr(a.err, QERR_BOUND);
+                        if (dir) lmb = min(lmb, lab);
+                        else lmf = min(lmf, lab);
+                    }
+                }
+                if (keep) ok = false;
+            }
+            uint32_t b = 0, cnt = 0;
+            if (ok) {
+                // out of the queue first, then its label: one lowered after
+                // this read queues the vertex again
+                atomicAnd(&queued[x], ~(1u << dir));
+                lab = __ldcg(dist + x);
+                const uint32_t *off = dir ? a.dn_off : a.up_off;
+                b = off[x];
+                const uint32_t e = off[x + 1];
+                if (b <= e && e <= (dir ? a.n_dn : a.n_up)) cnt = e - b;
+                else atomicOr(a.err, QERR_BOUND);
+            }
+            stat.exp += cnt ? 1u : 0u;
+            const uint32_t incl = warp_incl_scan(cnt);
+            if (lane == 31) q.wtot[warp] = incl;
+            q.beg[tid] = b;
+            q.lab[tid] = lab;
+            q.dir[tid] = (uint8_t)dir;
+            __syncthreads();
+            const uint32_t wt = q.wtot[lane];
+            const uint32_t wincl = warp_incl_scan(wt);
+            const uint32_t total = __shfl_sync(FULL, wincl, 31);
+            q.excl[tid] = __shfl_sync(FULL, wincl - wt, warp) + incl - cnt;
+            if (tid == 0) q.edges += total;
+            __syncthreads();
+            for (uint32_t e0 = tid; e0 < total; e0 += QD_THREADS) {
+                // owner entry: the largest k with excl[k] <= e0
+                uint32_t k = 0;
+#pragma unroll
+                for (uint32_t step = QD_THREADS / 2; step > 0; step >>= 1)
+                    if (q.excl[k + step] <= e0) k += step;
+                ++stat.edges;
+                const uint32_t edir = q.dir[k];
+                const uint2 e = (edir ? a.dn_adj : a.up_adj)[q.beg[k] + (e0 - q.excl[k])];
+                const uint32_t nd = sat_add(q.lab[k], e.y);
+                if (e.x >= a.n) {
+                    atomicOr(a.err, QERR_BOUND);
+                    continue;
+                }
+                if (nd == INF) continue;
+                if (PRUNE && nd >= *(volatile uint32_t *)&q.mu) continue;
+                uint32_t *ed = edir ? db : df;
+                if (nd >= __ldcg(ed + e.x)) continue;
+                const uint32_t old = atomicMin(&ed[e.x], nd);
+                if (nd >= old) continue;
+                if (old == INF) {
+                    const uint32_t p = atomicAdd(&q.nt, 1u);
+                    if (p < 2u * a.n) touched[p] = e.x;
+                    else atomicOr(a.err, QERR_BOUND);
+                }
+                if (edir) lmb = min(lmb, nd);
+                else lmf = min(lmf, nd);
+                if (PRUNE) {
+                    const uint32_t other = __ldcg((edir ? df : db) + e.x);
+                    if (other != INF) atomicMin(&q.mu, sat_add(nd, other));
+                }
+                if (!(atomicOr(&queued[e.x], 1u << edir) & (1u << edir))) {
+                    const uint32_t p = atomicAdd(ncnt, 1u);
+                    if (p < 2u * a.n) nxt[p] = e.x | (edir << 31);
+                    else atomicOr(a.err, QERR_BOUND);
+                }
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lmf = min(lmf, __shfl_xor_sync(FULL, lmf, o));
+            lmb = min(lmb, __shfl_xor_sync(FULL, lmb, o));
+        }
+        if (lane == 0) {
+            if (lmf != INF) atomicMin(&q.lmin3[(lvl + 1) % 3][0], lmf);
+            if (lmb != INF) atomicMin(&q.lmin3[(lvl + 1) % 3][1], lmb);
+        }
+    }
+    __syncthreads();
+    // the answer: the least meeting sum over the vertices reached
+    const uint32_t nt = min(q.nt, 2u * a.n);
+    if (tid == 0) q.mu = INF;
+    __syncthreads();
+    uint32_t mu = INF;
+    for (uint32_t p = tid; p < nt; p += QD_THREADS) {
+        const uint32_t v = __ldcg(touched + p);
+        mu = min(mu, sat_add(__ldcg(df + v), __ldcg(db + v)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mu = min(mu, __shfl_xor_sync(FULL, mu, o));
+    if (lane == 0 && mu != INF) atomicMin(&q.mu, mu);
+    __syncthreads();
+    mu_out = q.mu;
+    cnt_out = nt;
+    for (uint32_t p = tid; p < nt; p += QD_THREADS) {
+        const uint32_t v = __ldcg(touched + p);
+        df[v] = INF;
+        db[v] = INF;
+        queued[v] = 0;
+    }
+}
+
+// Query i's endpoints as ranks; false (in every thread), with the error
+// recorded and the answer INF, when an id is out of range.
+__device__ __forceinline__ bool query_ranks(const QArgs &a, uint32_t i, uint32_t &rs, uint32_t &rt) {
+    const uint32_t s = a.src ? a.src[i] : a.one_src, t = a.dst[i];
+    rs = s < a.n ? a.rank[s] : INF;
+    rt = t < a.n ? a.rank[t] : INF;
+    if (rs < a.n && rt < a.n) return true;
+    if (threadIdx.x == 0) {
+        atomicOr(a.err, s >= a.n || t >= a.n ? QERR_RANGE : QERR_BOUND);
+        a.out[i] = INF;
+        if (a.settled) a.settled[i] = 0;
+    }
+    return false;
+}
+
+template <bool PRUNE>
+__global__ void __launch_bounds__(QD_THREADS) k_query_dense(QArgs a, QDense dn) {
+    __shared__ QDSmem q;
+    const uint32_t tid = threadIdx.x;
+    pdl_wait();
     const uint32_t nitems = a.dense_first ? (uint32_t)a.k : a.work[a.ovf_cnt];
     QStat stat;
-    while (true) {
+    while (nitems) {
         __syncthreads();
         if (tid == 0) q.item = atomicAdd(&a.work[1], 1u);
         __syncthreads();
         if (q.item >= nitems) break;
         const uint32_t i = a.dense_first ? q.item : a.ovf[q.item];
-        const uint32_t s = i < a.k ? a.src[i] : INF, t = i < a.k ? a.dst[i] : INF;
-        const uint32_t rs = s < a.n ? a.rank[s] : INF, rt = t < a.n ? a.rank[t] : INF;
-        if (rs >= a.n || rt >= a.n) {
-            if (tid == 0) {
-                atomicOr(a.err, s >= a.n || t >= a.n ? QERR_RANGE : QERR_BOUND);
-                if (i < a.k) {
-                    a.out[i] = INF;
-                    if (a.settled) a.settled[i] = 0;
-                }
-            }
+        if (i >= a.k) {
+            if (tid == 0) atomicOr(a.err, QERR_BOUND);
             continue;
         }
+        uint32_t rs, rt, mu, cnt;
+        if (!query_ranks(a, i, rs, rt)) continue;
+        dense_query<PRUNE>(q, a, dn, rs, rt, mu, cnt, stat);
         if (tid == 0) {
-            df[rs] = 0;
-            db[rt] = 0;
-            queued[rs] = rs == rt ? 3u : 1u;
-            if (rs != rt) queued[rt] = 2u;
-            touched[0] = rs;
-            touched[1] = rt;
-            fra[0] = rs;
-            fra[1] = rt | 0x80000000u;
-            q.nt = 2;
-            q.mu = rs == rt ? 0u : INF;
-            q.cnt3[0] = 2;
-            q.cnt3[1] = 0;
-            q.lmin3[0][0] = q.lmin3[0][1] = 0;
-            q.lmin3[1][0] = q.lmin3[1][1] = INF;
-            q.delta = a.dense_delta;
-            q.edges = 0;
+            a.out[i] = mu;
+            if (a.settled) a.settled[i] = cnt;
         }
-        for (uint32_t lvl = 0;; ++lvl) {
-            __syncthreads();
-            const uint32_t nfront = q.cnt3[lvl % 3];
-            const uint32_t mu0 = q.mu, minf = q.lmin3[lvl % 3][0], minb = q.lmin3[lvl % 3][1];
-            uint32_t delta = q.delta;
-            const uint32_t did = q.edges;
-            if (nfront == 0) break;
-            if (lvl >= (1u << 30)) {  // the least label grows every other level at the latest
-                if (tid == 0) atomicOr(a.err, QERR_BOUND);
-                break;
-            }
-            if (lvl && did < QD_EDGES_LOW) delta = min(2u * delta, 1u << 30);
-            else if (did > QD_EDGES_HIGH) delta = max(delta / 2u, 1u);
-            const uint32_t thrf = sat_add(minf, delta), thrb = sat_add(minb, delta);
-            __syncthreads();
-            if (tid == 0) {
-                q.cnt3[(lvl + 2) % 3] = 0;
-                q.lmin3[(lvl + 2) % 3][0] = q.lmin3[(lvl + 2) % 3][1] = INF;
-                q.delta = delta;
-                q.edges = 0;
-            }
-            const uint32_t *cur = lvl & 1u ? frb : fra;
-            uint32_t *nxt = lvl & 1u ? fra : frb;
-            uint32_t *ncnt = &q.cnt3[(lvl + 1) % 3];
-            uint32_t lmf = INF, lmb = INF;  // least labels this thread queues
-            for (uint32_t t0 = 0; t0 < nfront; t0 += QD_THREADS) {
-                const uint32_t fi = t0 + tid;
-                const uint32_t ent = fi < nfront ? __ldcg(cur + fi) : 0;
-                const uint32_t x = ent & 0x7FFFFFFFu, dir = ent >> 31;
-                bool ok = fi < nfront && x < a.n;
-                if (fi < nfront && !ok) atomicOr(a.err, QERR_BOUND);
-                uint32_t *dist = dir ? db : df;
-                uint32_t lab = ok ? __ldcg(dist + x) : INF;
-                bool keep = false;
-                if (PRUNE) {
-                    const bool drop = ok && (lab >= mu0 || (x >= a.core_first &&
-                                                            sat_add(lab, dir ? minf : minb) >= mu0));
-                    keep = ok && !drop && lab > (dir ? thrb : thrf);
-                    if (drop) {
-                        // a label lowered meanwhile is queued again
-                        atomicAnd(&queued[x], ~(1u << dir));
-                        const uint32_t now = __ldcg(dist + x);
-                        if (now < lab) {
-                            lab = now;
-                            if (!(atomicOr(&queued[x], 1u << dir) & (1u << dir))) keep = true;
-                        }
-                        ok = false;
-                    }
-                    const uint32_t m = __ballot_sync(FULL, keep);
-                    if (m) {
-                        uint32_t p = 0;
-                        const uint32_t leader = __ffs(m) - 1;
-                        if (lane == leader) p = atomicAdd(ncnt, (uint32_t)__popc(m));
-                        p = __shfl_sync(FULL, p, leader) + __popc(m & ((1u << lane) - 1u));
-                        if (keep) {
-                            if (p < 2u * a.n) nxt[p] = ent;
-                            else atomicOr(a.err, QERR_BOUND);
-                            if (dir) lmb = min(lmb, lab);
-                            else lmf = min(lmf, lab);
-                        }
-                    }
-                    if (keep) ok = false;
-                }
-                uint32_t b = 0, cnt = 0;
-                if (ok) {
-                    // out of the queue first, then its label: one lowered after
-                    // this read queues the vertex again
-                    atomicAnd(&queued[x], ~(1u << dir));
-                    lab = __ldcg(dist + x);
-                    const uint32_t *off = dir ? a.dn_off : a.up_off;
-                    b = off[x];
-                    const uint32_t e = off[x + 1];
-                    if (b <= e && e <= (dir ? a.n_dn : a.n_up)) cnt = e - b;
-                    else atomicOr(a.err, QERR_BOUND);
-                }
-                stat.exp += cnt ? 1u : 0u;
-                const uint32_t incl = warp_incl_scan(cnt);
-                if (lane == 31) q.wtot[warp] = incl;
-                q.beg[tid] = b;
-                q.lab[tid] = lab;
-                q.dir[tid] = (uint8_t)dir;
-                __syncthreads();
-                const uint32_t wt = q.wtot[lane];
-                const uint32_t wincl = warp_incl_scan(wt);
-                const uint32_t total = __shfl_sync(FULL, wincl, 31);
-                q.excl[tid] = __shfl_sync(FULL, wincl - wt, warp) + incl - cnt;
-                if (tid == 0) q.edges += total;
-                __syncthreads();
-                for (uint32_t e0 = tid; e0 < total; e0 += QD_THREADS) {
-                    // owner entry: the largest k with excl[k] <= e0
-                    uint32_t k = 0;
-#pragma unroll
-                    for (uint32_t step = QD_THREADS / 2; step > 0; step >>= 1)
-                        if (q.excl[k + step] <= e0) k += step;
-                    ++stat.edges;
-                    const uint32_t edir = q.dir[k];
-                    const uint2 e = (edir ? a.dn_adj : a.up_adj)[q.beg[k] + (e0 - q.excl[k])];
-                    const uint32_t nd = sat_add(q.lab[k], e.y);
-                    if (e.x >= a.n) {
-                        atomicOr(a.err, QERR_BOUND);
-                        continue;
-                    }
-                    if (nd == INF) continue;
-                    if (PRUNE && nd >= *(volatile uint32_t *)&q.mu) continue;
-                    uint32_t *ed = edir ? db : df;
-                    if (nd >= __ldcg(ed + e.x)) continue;
-                    const uint32_t old = atomicMin(&ed[e.x], nd);
-                    if (nd >= old) continue;
-                    if (old == INF) {
-                        const uint32_t p = atomicAdd(&q.nt, 1u);
-                        if (p < 2u * a.n) touched[p] = e.x;
-                        else atomicOr(a.err, QERR_BOUND);
-                    }
-                    if (edir) lmb = min(lmb, nd);
-                    else lmf = min(lmf, nd);
-                    if (PRUNE) {
-                        const uint32_t other = __ldcg((edir ? df : db) + e.x);
-                        if (other != INF) atomicMin(&q.mu, sat_add(nd, other));
-                    }
-                    if (!(atomicOr(&queued[e.x], 1u << edir) & (1u << edir))) {
-                        const uint32_t p = atomicAdd(ncnt, 1u);
-                        if (p < 2u * a.n) nxt[p] = e.x | (edir << 31);
-                        else atomicOr(a.err, QERR_BOUND);
-                    }
-                }
-                __syncthreads();
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                lmf = min(lmf, __shfl_xor_sync(FULL, lmf, o));
-                lmb = min(lmb, __shfl_xor_sync(FULL, lmb, o));
-            }
-            if (lane == 0) {
-                if (lmf != INF) atomicMin(&q.lmin3[(lvl + 1) % 3][0], lmf);
-                if (lmb != INF) atomicMin(&q.lmin3[(lvl + 1) % 3][1], lmb);
-            }
+    }
+    if (nitems) qb_flush_stat(stat, a.stats);
+    // The last block to finish leaves the batch's counters at zero for the
+    // next batch. (Every block has read the overflow count before it counts
+    // itself finished.)
+    __syncthreads();
+    if (tid == 0 && atomicAdd(&a.work[a.ticket], 1u) + 1 == gridDim.x)
+        for (uint32_t w = 0; w <= a.ticket; ++w) a.work[w] = 0;
+}
+
+// Small batches: a block of 1024 threads a query, in one launch; queries that
+// outgrow the table are left to the dense kernel behind it. With that few
+// queries the time of one counts: the chain of round trips of its levels, and
+// how fast one SM issues their instructions. The levels are block_search's,
+// with stalling and buckets, but a warp takes whole rows: a level's entries
+// are dealt to 32 warps, most of which hold one or two, and each row's lanes
+// read its stall edges and its out-edges together, without the scans and owner
+// searches of flattened rows. An entry found stalled drops the out-edges it has
+// read. Geometric graph of 1M vertices: 69 us a query alone, 114 for 152 at
+// once, against 122 and 216 by the launches that larger batches take. (Rows
+// flattened over the whole block: 80 and 133 us. Whole rows in the blocks of
+// 256 threads that larger batches use, several rows a warp: slower, 302 us for
+// 777 queries against 254.)
+constexpr int QS_THREADS = 1024;
+
+template <int TB>
+__device__ bool row_search(QBSmem<TB> &q, const QArgs &a, QStat &stat) {
+    constexpr uint32_t FC = QBSmem<TB>::FC, CW = QBSmem<TB>::CW;
+    const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    constexpr uint32_t W = QS_THREADS / 32;
+    for (uint32_t lvl = 1;; ++lvl) {
+        __syncthreads();
+        const uint32_t cur = (lvl - 1) & 1u;
+        const uint32_t nfront = q.cnt3[(lvl - 1) % 3];
+        const uint32_t ovf = q.ovf;
+        if (ovf) return false;
+        if (nfront == 0) return true;
+        if (lvl >= 0xFFFFu) {
+            if (tid == 0) atomicOr(a.err, QERR_BOUND);
+            return false;
         }
-        __syncthreads();
-        // the answer: the least meeting sum over the vertices reached
-        const uint32_t nt = min(q.nt, 2u * a.n);
-        if (tid == 0) q.mu = INF;
-        __syncthreads();
-        uint32_t mu = INF;
-        for (uint32_t p = tid; p < nt; p += QD_THREADS) {
-            const uint32_t v = __ldcg(touched + p);
-            mu = min(mu, sat_add(__ldcg(df + v), __ldcg(db + v)));
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mu = min(mu, __shfl_xor_sync(FULL, mu, o));
-        if (lane == 0 && mu != INF) atomicMin(&q.mu, mu);
-        __syncthreads();
+        const uint32_t thr_f = sat_add(q.lmin3[(lvl - 1) % 3][0], a.delta),
+                       thr_b = sat_add(q.lmin3[(lvl - 1) % 3][1], a.delta);
         if (tid == 0) {
-            a.out[i] = q.mu;
-            if (a.settled) a.settled[i] = nt;
+            q.cnt3[(lvl + 1) % 3] = 0;
+            q.lmin3[(lvl + 1) % 3][0] = q.lmin3[(lvl + 1) % 3][1] = INF;
         }
-        for (uint32_t p = tid; p < nt; p += QD_THREADS) {
-            const uint32_t v = __ldcg(touched + p);
-            df[v] = INF;
-            db[v] = INF;
-            queued[v] = 0;
+        for (uint32_t j = tid; j < 2u * CW; j += QS_THREADS) (&q.claim[(lvl + 1) & 1u][0][0])[j] = 0;
+        const uint32_t nxt_cnt = lvl % 3;
+        uint32_t *next_front = q.front[cur ^ 1u];
+        uint32_t lmf = INF, lmb = INF;
+        for (uint32_t p0 = 0; p0 + warp < nfront; p0 += QS_THREADS) {
+            const uint32_t fi = p0 + warp + W * lane;
+            bool fv = fi < nfront && fi < FC;
+            const uint32_t ent = fv ? q.front[cur][fi] : 0;
+            const uint32_t dir = ent >> 31, slot = ent & 0x7FFFFFFFu;
+            const uint32_t lab = fv && slot < QBSmem<TB>::T ? (dir ? q.db[slot] : q.df[slot]) : INF;
+            if (fv && lab >= q.mu) {
+                fv = false;  // cannot improve the answer
+            } else if (fv && lab > (dir ? thr_b : thr_f)) {
+                // stays queued
+                if (qb_claim(q, slot, dir, lvl)) {
+                    const uint32_t p = atomicAdd(&q.cnt3[nxt_cnt], 1u);
+                    if (p < FC) next_front[p] = ent;
+                    else q.ovf = 1;
+                    if (dir) lmb = min(lmb, lab);
+                    else lmf = min(lmf, lab);
+                }
+                fv = false;
+            }
+            uint32_t b, cnt, dx, sb, se;
+            qb_entry_both(q, a, fv, ent, b, cnt, dx, sb, se);
+            uint32_t scnt = 0;
+            if (cnt && sb <= se && se <= (dir ? a.n_up : a.n_dn)) scnt = se - sb;
+            else if (cnt) atomicOr(a.err, QERR_BOUND);
+            stat.exp += cnt ? 1u : 0u;
+            stat.edges += scnt;
+            for (uint32_t m = __ballot_sync(FULL, cnt != 0); m; m &= m - 1) {
+                const uint32_t o = __ffs(m) - 1;
+                const uint32_t ob = __shfl_sync(FULL, b, o), oc = __shfl_sync(FULL, cnt, o),
+                               od = __shfl_sync(FULL, dx, o), osb = __shfl_sync(FULL, sb, o),
+                               osc = __shfl_sync(FULL, scnt, o), odir = __shfl_sync(FULL, ent, o) >> 31;
+                const uint2 *oadj = (odir ? a.dn_adj : a.up_adj) + ob, *sadj = (odir ? a.up_adj : a.dn_adj) + osb;
+                uint2 y = lane < oc ? oadj[lane] : make_uint2(0, 0);
+                bool stalled = false;
+                for (uint32_t j = lane; j < osc; j += 32) {
+                    const uint2 z = sadj[j];
+                    const uint32_t at = z.x < a.n ? qb_find<TB>(q.key, z.x) : EMPTY;
+                    stalled |= at != EMPTY && sat_add(odir ? q.db[at] : q.df[at], z.y) < od;
+                }
+                if (__any_sync(FULL, stalled)) continue;
+                stat.edges += lane == 0 ? oc : 0;
+                for (uint32_t j = lane; j < oc;) {
+                    qb_relax<true, TB, true>(q, a, odir, y, od, lvl, nxt_cnt, next_front, lmf, lmb);
+                    j += 32;
+                    if (j < oc) y = oadj[j];
+                }
+            }
         }
+        lmf = __reduce_min_sync(FULL, lmf);
+        lmb = __reduce_min_sync(FULL, lmb);
+        if (lane == 0) {
+            if (lmf != INF) atomicMin(&q.lmin3[nxt_cnt][0], lmf);
+            if (lmb != INF) atomicMin(&q.lmin3[nxt_cnt][1], lmb);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(QS_THREADS, 1) k_query_small(QArgs a) {
+    extern __shared__ __align__(16) unsigned char qb_raw[];
+    QBSmem<12> &q = *reinterpret_cast<QBSmem<12> *>(qb_raw);
+    QStat stat;
+    pdl_launch();
+    qb_clear(q);
+    for (uint32_t i = blockIdx.x; i < a.k; i += gridDim.x) {
+        uint32_t rs, rt, mu, cnt;
+        if (!query_ranks(a, i, rs, rt)) continue;
+        if (!block_query_by(q, a, rs, rt, mu, cnt, [&] { return row_search<12>(q, a, stat); })) {
+            if (threadIdx.x == 0) a.ovf[atomicAdd(&a.work[a.ovf_cnt], 1u)] = i;
+            continue;
+        }
+        if (threadIdx.x == 0) a.out[i] = mu;
     }
     qb_flush_stat(stat, a.stats);
 }
@@ -367,6 +514,7 @@ void qb_resolve(int s) {
 void qb_resolve_occupancy() {
     if (g_qb_bps[0][0][0] >= 0) return;
     qb_resolve<12>(0);
+    CH_CUDA_TRY(cudaFuncSetAttribute(k_query_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(QBSmem<12>)));
     qb_resolve<11>(1);
 }
 
@@ -427,7 +575,8 @@ void query_init(ch_s *h) {
     const uint32_t n = h->n;
     h->qerr.alloc(1);
     h->qerr.zero(0);
-    h->qwork.alloc(8);
+    h->qwork.alloc(QWORK);
+    h->qwork.zero(0);
     h->q_ovf_cap = Q_CHUNK;
     h->q_ovf_list.alloc(2 * Q_CHUNK);  // overflow lists of the two block-kernel passes
     // as many slots as the chip runs blocks of the dense kernel at once (two
@@ -513,16 +662,49 @@ QArgs hierarchy_args(const ch_s *h) {
 void launch_query_dense(const ch_s *h, const QArgs &a, bool prune, uint64_t k, cudaStream_t st) {
     const QDense dn = dense_slots(h);
     const unsigned blocks = (unsigned)std::min<uint64_t>(dn.nslots, k);
-    if (prune) k_query_dense<true><<<blocks, QD_THREADS, 0, st>>>(a, dn);
-    else k_query_dense<false><<<blocks, QD_THREADS, 0, st>>>(a, dn);
+    launch_pdl(prune ? k_query_dense<true> : k_query_dense<false>, blocks, QD_THREADS, 0, st, a, dn);
+}
+
+}  // namespace
+
+namespace {
+
+// A batch with at most one query an SM is small: two of its 1024-thread
+// blocks do not fit an SM (60 registers a thread), and at two queries an SM
+// both ways take the same time (1M vertices, 304 queries: 182 and 212 us; 256K
+// vertices: 126 and 120 us). Not for queries that need the dense kernel.
+bool small_batch(const QArgs &a, uint64_t k) { return k <= (uint64_t)device_sm_count() && !a.dense_first; }
+
+void launch_query_small(const QArgs &a, cudaStream_t st) {
+    k_query_small<<<(unsigned)a.k, QS_THREADS, sizeof(QBSmem<12>), st>>>(a);
     CH_CHECK_LAUNCH();
 }
 
 }  // namespace
 
+bool query_batch_small(ch_s *h, const uint32_t *src, uint32_t one_src, const uint32_t *dst, uint64_t k,
+                       uint32_t *dist_out, cudaStream_t st) {
+    QArgs a = hierarchy_args(h);
+    if (!small_batch(a, k)) return false;
+    a.src = src;
+    a.one_src = one_src;
+    a.dst = dst;
+    a.out = dist_out;
+    a.settled = nullptr;
+    a.k = k;
+    a.work = h->qwork.ptr;
+    a.ticket = QWORK - 1;
+    a.ovf = h->q_ovf_list.ptr;
+    a.ovf_cnt = 2;
+    launch_query_small(a, st);
+    launch_query_dense(h, a, true, k, st);
+    return true;
+}
+
 void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
                  uint32_t *dist_out, uint32_t *settled_out, cudaStream_t st, bool searches_only) {
     if (k == 0) return;
+    if (!settled_out && !searches_only && query_batch_small(h, src, 0, dst, k, dist_out, st)) return;
     for (uint64_t c0 = 0; c0 < k; c0 += Q_CHUNK) {
         const uint64_t kc = std::min<uint64_t>(Q_CHUNK, k - c0);
         QArgs a = hierarchy_args(h);
@@ -532,9 +714,9 @@ void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
         a.settled = settled_out ? settled_out + c0 : nullptr;
         a.k = kc;
         a.work = h->qwork.ptr;
+        a.ticket = QWORK - 1;
         a.in_list = nullptr;
         a.in_cnt = 0;
-        CH_CUDA_TRY(cudaMemsetAsync(h->qwork.ptr, 0, 8 * sizeof(uint32_t), st));
         // Pruned searches unless the caller asked for search-space sizes,
         // which are defined by the exhaustive upward searches.
         const bool prune = settled_out == nullptr;
@@ -792,7 +974,7 @@ void query_graph_free(ch_query_graph_s *g) {
 
 namespace {
 
-constexpr uint32_t kStaticScratchHead = 4;  // [0] block counter, [1] dense counter, [2] overflow count
+constexpr uint32_t kStaticScratchHead = 4;  // [0] block counter, [1] dense counter, [2] overflow count, [3] finished blocks
 __device__ __align__(256) uint32_t g_static_query_scratch[kStaticScratchHead + CH_STATIC_QUERY_MAX];
 
 std::mutex g_static_mu;
@@ -838,10 +1020,10 @@ void query_batch_static(ch_s *h, const uint32_t *src, const uint32_t *dst, uint6
     a.ctr = 0;
     a.ovf = scratch + kStaticScratchHead;
     a.ovf_cnt = 2;
-    // the counters keep the previous call's values: clear them
-    CH_CUDA_TRY(cudaMemsetAsync(scratch, 0, kStaticScratchHead * sizeof(uint32_t), st));
+    a.ticket = kStaticScratchHead - 1;
     // one block-kernel pass (large tables): the scratch holds one list
-    if (!a.dense_first) launch_query_block(h, a, true, false, k, st);
+    if (small_batch(a, k)) launch_query_small(a, st);
+    else if (!a.dense_first) launch_query_block(h, a, true, false, k, st);
     launch_query_dense(h, a, true, k, st);
 }
 
