@@ -291,8 +291,8 @@ int ch_query_one_to_many(ch_t *ch, uint32_t s, const uint32_t *dst, uint64_t k,
  * dist_out[i * n + v] = length of a shortest path src[i] -> v in the input
  * graph, for every vertex v (0xFFFFFFFF if unreachable). src (uint32[k]) and
  * dist_out (uint32[k * n], row-major, caller-owned) are DEVICE pointers; the
- * work is enqueued on `stream`. The sweeps run over the rank order, 16
- * sources at a time, in library-owned scratch of 64 bytes per vertex, so
+ * work is enqueued on `stream`. The sweeps run over the rank order, up to 64
+ * sources at a time, in library-owned scratch of up to 256 bytes per vertex, so
  * calls on one handle must not overlap on the GPU. A hierarchy with a core
  * iterates the core on the host's command, so the call then waits for
  * `stream` once per core pass. Ids >= n are reported by ch_query_status as

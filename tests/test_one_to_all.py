@@ -51,6 +51,35 @@ def test_geometric_ragged_batches(k):
     assert np.array_equal(got, och.one_to_all(src))
 
 
+@pytest.mark.parametrize("k", [2, 4, 5, 70])
+def test_more_small_levels_than_shared_memory_holds(k):
+    # ids break ties on a unit chain in order: thousands of levels of a vertex
+    # or two, of which the block that walks the top holds the last 16,000 ranks
+    g = I.chain_graph(17_500, wmin=1, wmax=1)
+    ch = _ch()
+    h = ch.CH.build(g, hop_limit=2, tie_break=ch.CH_TIE_ID)
+    src = np.random.default_rng(k).integers(0, g.n, k).astype(np.uint32)
+    got = _run(h, src)
+    want = np.abs(np.arange(g.n)[None, :] - src.astype(np.int64)[:, None])
+    assert np.array_equal(got, want)
+
+
+def test_source_that_climbs_to_thousands_at_once():
+    # an extra vertex with no in-edge (so contracted first) and 3,000
+    # out-edges: more than a step of the climb queues
+    g = I.geometric_knn_graph(10_000, seed=132)
+    rng = np.random.default_rng(133)
+    src, dst, w = g.edges()
+    to = rng.choice(g.n, 3000, replace=False)
+    g = I.csr_from_edges(g.n + 1, np.concatenate([src, np.full(3000, g.n)]), np.concatenate([dst, to]),
+                         np.concatenate([w, rng.integers(1, 100, 3000)]))
+    h = _ch().CH.build(g, hop_limit=5)
+    sources = np.array([g.n - 1, 5, g.n - 1, 77], np.uint32)
+    got = _run(h, sources)
+    for i, s in enumerate(sources.tolist()):
+        assert np.array_equal(got[i], O.dijkstra(g, s))
+
+
 def test_rmat_with_a_core_and_a_loaded_hierarchy(tmp_path):
     g = I.rmat_graph(scale=12, nsamples=1 << 15, wmax=1000, seed=91)
     h = _ch().CH.build(g, hop_limit=5, max_candidates_per_vertex=16)
