@@ -102,7 +102,7 @@ struct Ctl {
     unsigned long long dm_count;     // keys in the memoised-distance map since its last clear
     unsigned long long pruned;       // overlay edges pruned this round
     uint32_t nDirty;                 // vertices whose lists hold pruned entries
-    uint32_t longRows;               // rank-ordered CSR rows left for the radix sort
+    uint32_t longRows[2], longest[2];  // rank-ordered CSR rows left unsorted, per direction, and the longest
     // shortcut log entries so far (device-side, so that k_insert needs no
     // host value), and the contraction counters of the last finished round,
     // copied by k_round_end for the host's next read
@@ -1882,13 +1882,22 @@ __global__ void k_orig_deg(Dev d) {
 // Step 3: select strict local minima of the key
 // --------------------------------------------------------------------------
 
-__global__ void k_select(Dev d, const uint32_t *VO, uint32_t nVO, uint32_t r, uint32_t *F) {
+// A warp takes `per` vertices and spreads their neighbour lists over its lanes;
+// `per` is 32 while there are many live vertices and falls to 1 with them, so
+// that the last hundreds of rounds, whose lists are the longest, still use the
+// whole chip (1,000 vertices of degree 50: 22 -> 8 us). Vertices that are
+// not eligible have nothing to compare, and a list above SELECT_LONG is walked
+// by itself until a neighbour beats it: hubs nearly always fall at the first
+// step (a round of an RMAT 2^17 build: 2.7 -> 0.06 ms).
+constexpr uint32_t SELECT_LONG = 256;
+
+__global__ void k_select(Dev d, const uint32_t *VO, uint32_t nVO, uint32_t per, uint32_t r, uint32_t *F) {
     const uint32_t lane = lane_id();
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t base = warp * 32; base < nVO; base += nwarps * 32) {
+    for (uint32_t base = warp * per; base < nVO; base += nwarps * per) {
         const uint32_t i = base + lane;
-        const bool valid = i < nVO;
+        const bool valid = lane < per && i < nVO;
         const uint32_t u = valid ? VO[i] : 0;
         const bool uok = valid && id_ok(d, u);
         const uint64_t ku = uok ? select_key(d, u) : 0;
@@ -1896,11 +1905,30 @@ __global__ void k_select(Dev d, const uint32_t *VO, uint32_t nVO, uint32_t r, ui
         const uint64_t ib = uok ? d.in_beg[u] : 0;
         const uint32_t od = (uok && out_list_ok(d, ob, d.out_deg[u])) ? d.out_deg[u] : 0;
         const uint32_t id = (uok && in_list_ok(d, ib, d.in_deg[u])) ? d.in_deg[u] : 0;
-        const uint32_t c = od + id;
+        const bool cand = uok && !d.inel[u];
+        const bool lng = cand && od + id > SELECT_LONG;
+        const uint32_t c = cand && !lng ? od + id : 0;
         const uint32_t incl = warp_incl_scan(c);
         const uint32_t total = __shfl_sync(FULL, incl, 31);
         const uint32_t excl = incl - c;
         bool beaten = false;
+        for (uint32_t m = __ballot_sync(FULL, lng); m; m &= m - 1) {
+            const uint32_t o = __ffs(m) - 1;
+            const uint32_t od_o = __shfl_sync(FULL, od, o), c_o = od_o + __shfl_sync(FULL, id, o);
+            const uint64_t ob_o = __shfl_sync(FULL, ob, o), ib_o = __shfl_sync(FULL, ib, o),
+                           ku_o = __shfl_sync(FULL, ku, o);
+            bool hit = false;
+            for (uint32_t j0 = 0; j0 < c_o && !hit; j0 += 32) {
+                const uint32_t jj = j0 + lane;
+                bool bt = false;
+                if (jj < c_o) {
+                    const uint32_t nb = jj < od_o ? d.out_adj[ob_o + jj].x : d.in_adj[ib_o + (jj - od_o)].x;
+                    bt = id_ok(d, nb) && select_key(d, nb) < ku_o;
+                }
+                hit = __any_sync(FULL, bt);
+            }
+            if (lane == o && hit) beaten = true;
+        }
         for (uint32_t b = 0; b < total; b += 32) {
             const uint32_t idx = b + lane;
             const uint32_t o = warp_owner(excl, idx);
@@ -1919,7 +1947,7 @@ __global__ void k_select(Dev d, const uint32_t *VO, uint32_t nVO, uint32_t r, ui
             const uint32_t lo = max(excl, b), hi = min(excl + c, b + 32);
             if (hi > lo && (B & lane_bits(lo - b, hi - b))) beaten = true;
         }
-        const bool sel = uok && !beaten && !d.inel[u];
+        const bool sel = cand && !beaten;
         if (sel) d.level[u] = r;
         const uint32_t pos = warp_append(sel, &d.ctl->nF);
         if (sel) F[pos] = u;
@@ -2389,6 +2417,42 @@ __global__ void k_ranked_deg(const uint32_t *perm, uint32_t n, const uint32_t *d
 }
 
 constexpr uint32_t RANKED_SORT_MAX = 64;  // longest row a thread insertion-sorts
+constexpr uint32_t ROW_SORT_MAX = 16384;  // longest row a block sorts in shared memory (8 B an entry)
+constexpr int ROW_SORT_THREADS = 512;
+
+// Sorts the listed rows of a rank-ordered CSR by target rank, a block a row: a
+// bitonic sort in shared memory of target << 32 | weight (targets of a row are
+// distinct), padded to a power of two with ones. Rows above ROW_SORT_MAX are
+// left. An RMAT 2^17 hierarchy (5.3M entries in both CSRs, rows of up to 10^4):
+// well under 1 ms, against 6.3 for a radix sort of both whole CSRs.
+__global__ void __launch_bounds__(ROW_SORT_THREADS)
+k_sort_rows(const uint32_t *rows, const uint32_t *off, uint2 *adj) {
+    extern __shared__ unsigned long long row_smem[];
+    const uint32_t i = rows[blockIdx.x];
+    const uint32_t b = off[i], m = off[i + 1] - b;
+    if (m > ROW_SORT_MAX) return;
+    uint32_t n2 = 2;
+    while (n2 < m) n2 <<= 1;
+    for (uint32_t j = threadIdx.x; j < n2; j += ROW_SORT_THREADS) {
+        const uint2 a = j < m ? adj[b + j] : make_uint2(INF, INF);
+        row_smem[j] = ((unsigned long long)a.x << 32) | a.y;
+    }
+    for (uint32_t size = 2; size <= n2; size <<= 1)
+        for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+            __syncthreads();
+            for (uint32_t t = threadIdx.x; t < n2 / 2; t += ROW_SORT_THREADS) {
+                const uint32_t lo = 2 * t - (t & (stride - 1)), hi = lo + stride;
+                const unsigned long long x = row_smem[lo], y = row_smem[hi];
+                if ((x > y) == ((lo & size) == 0)) {
+                    row_smem[lo] = y;
+                    row_smem[hi] = x;
+                }
+            }
+        }
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < m; j += ROW_SORT_THREADS)
+        adj[b + j] = make_uint2((uint32_t)(row_smem[j] >> 32), (uint32_t)row_smem[j]);
+}
 
 // Keys of every entry of a rank-ordered CSR for the radix sort of its rows:
 // row << 32 | target rank (one warp per row), the weight as the value.
@@ -2415,7 +2479,7 @@ __global__ void k_row_unpack(const uint64_t *keys, const uint32_t *vals, uint64_
 __global__ void k_ranked_fill(const uint32_t *perm, const uint32_t *rank, uint32_t n,
                               const uint64_t *beg, const uint32_t *deg, const uint2 *src,
                               uint64_t src_count, const uint32_t *off, uint64_t dst_count,
-                              uint2 *dst, Ctl *ctl) {
+                              uint2 *dst, uint32_t dir, uint32_t *rows, Ctl *ctl) {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const uint32_t v = perm[i];
         if (v >= n) {
@@ -2439,10 +2503,11 @@ __global__ void k_ranked_fill(const uint32_t *perm, const uint32_t *rank, uint32
             out[j] = make_uint2(rank[e.x], e.y);
         }
         // rows are sorted by target rank, which makes the list order
-        // canonical: short rows here (insertion sort), longer ones by the
-        // radix sort of the whole CSR that a set flag asks for
+        // canonical: short rows here (insertion sort), longer ones are listed
+        // for k_sort_rows or, above what a block sorts, for the radix sort
         if (dg > RANKED_SORT_MAX) {
-            ctl->longRows = 1;
+            rows[atomicAdd(&ctl->longRows[dir], 1u)] = i;
+            atomicMax(&ctl->longest[dir], dg);
             continue;
         }
         for (uint32_t j = 1; j < dg; ++j) {
@@ -2880,7 +2945,10 @@ void Builder::run_rounds() {
         mark(&h->t_score_ms, e0, 0);
         // 3: select
         e0 = start();
-        k_select<<<grid_for((uint64_t)nVO, 256, sms * 8), 256, 0, st>>>(d, VO.ptr, nVO, r, F.ptr);
+        // about 16 warps an SM before a warp takes a second vertex
+        const uint32_t per = (uint32_t)std::min<uint64_t>(32, 1 + nVO / (16 * (uint64_t)sms));
+        k_select<<<grid_for((uint64_t)(nVO + per - 1) / per * 32, 256, sms * 8), 256, 0, st>>>(d, VO.ptr, nVO, per,
+                                                                                              r, F.ptr);
         CH_CHECK_LAUNCH();
         mark(&h->t_select_ms, e0, 1);
         // 4: contraction bookkeeping
@@ -3031,6 +3099,8 @@ void Builder::postprocess() {
         throw Error{CH_ERANGE, "hierarchy has 2^32 - 1 or more edges in one direction"};
     h->n_up = n_up;
     h->n_down = n_dn;
+    DevBuf<uint32_t> rows;  // unsorted rows of each direction
+    rows.alloc(2 * (size_t)n);
     for (int dir = 0; dir < 2; ++dir) {
         DevBuf<uint32_t> &off = dir == 0 ? h->up_off : h->dn_off;
         DevBuf<uint2> &adj = dir == 0 ? h->up_adj : h->dn_adj;
@@ -3045,21 +3115,29 @@ void Builder::postprocess() {
                                           dir == 0 ? ch_up_deg.ptr : ch_dn_deg.ptr,
                                           dir == 0 ? ch_up.ptr : ch_dn.ptr,
                                           dir == 0 ? hctl->ch_up_tail : hctl->ch_dn_tail, off.ptr,
-                                          dir == 0 ? n_up : n_dn, adj.ptr, ctl.ptr);
+                                          dir == 0 ? n_up : n_dn, adj.ptr, (uint32_t)dir,
+                                          rows.ptr + (size_t)dir * n, ctl.ptr);
         CH_CHECK_LAUNCH();
     }
     sync_ctl();
-    if (hctl->longRows) {
-        // some row is longer than a thread sorts: sort every row of both
-        // CSRs at once by (row, target rank)
-        std::vector<int> rd;
-        append_digits(rd, 0, bits_for(n));
-        append_digits(rd, 32, bits_for(n));
-        for (int dir = 0; dir < 2; ++dir) {
-            DevBuf<uint32_t> &off = dir == 0 ? h->up_off : h->dn_off;
-            DevBuf<uint2> &adj = dir == 0 ? h->up_adj : h->dn_adj;
-            const uint64_t m = dir == 0 ? n_up : n_dn;
-            if (m < 2) continue;
+    for (int dir = 0; dir < 2; ++dir) {
+        DevBuf<uint32_t> &off = dir == 0 ? h->up_off : h->dn_off;
+        DevBuf<uint2> &adj = dir == 0 ? h->up_adj : h->dn_adj;
+        const uint64_t m = dir == 0 ? n_up : n_dn;
+        if (!hctl->longRows[dir]) continue;
+        if (hctl->longest[dir] <= ROW_SORT_MAX) {
+            uint32_t n2 = 2;
+            while (n2 < hctl->longest[dir]) n2 <<= 1;
+            const int smem = (int)(n2 * sizeof(unsigned long long));
+            CH_CUDA_TRY(cudaFuncSetAttribute(k_sort_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            k_sort_rows<<<hctl->longRows[dir], ROW_SORT_THREADS, smem, st>>>(rows.ptr + (size_t)dir * n, off.ptr,
+                                                                             adj.ptr);
+            CH_CHECK_LAUNCH();
+        } else {
+            // sort every row of the CSR at once by (row, target rank)
+            std::vector<int> rd;
+            append_digits(rd, 0, bits_for(n));
+            append_digits(rd, 32, bits_for(n));
             DevBuf<uint64_t> k1, k2;
             DevBuf<uint32_t> v1, v2;
             k1.alloc(m);
@@ -3075,6 +3153,7 @@ void Builder::postprocess() {
             CH_CUDA_TRY(cudaStreamSynchronize(st));
         }
     }
+    CH_CUDA_TRY(cudaStreamSynchronize(st));  // before `rows` goes
 }
 
 }  // namespace

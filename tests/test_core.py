@@ -250,3 +250,21 @@ def test_core_table_label_placements(n, seed):
     gch.core_table()
     s, t = I.random_pairs(g.n, 300, seed=seed)
     assert np.array_equal(gch.query(s, t), O.dijkstra_pairs(g, s, t))
+
+
+# Rows of the rank-ordered CSRs: insertion-sorted by a thread up to 64 entries,
+# by a block up to 16,384, by a radix sort above. A star whose vertices all stay
+# in the core has one row of its leaves in both directions.
+@pytest.mark.parametrize("leaves", [64, 65, 1000, 16_384, 16_385])
+def test_long_rows(leaves):
+    g = I.star_graph(leaves, wmax=1000, seed=leaves)
+    gch = _ch().CH.build(g, hop_limit=5, max_candidates_per_vertex=0)
+    assert gch.stats()["core_vertices"] == g.n
+    ex = gch.export()
+    src, dst, w = g.edges()
+    want = np.stack([src, dst, w], 1).astype(np.uint32)
+    for key, rows in (("up", want), ("down", want)):
+        got = ex[key]
+        assert np.array_equal(got[np.lexsort(got.T[::-1])], rows[np.lexsort(rows.T[::-1])]), key
+    s, t = I.random_pairs(g.n, 200, seed=leaves)
+    assert np.array_equal(gch.query(s, t), O.dijkstra_pairs(g, s, t))
