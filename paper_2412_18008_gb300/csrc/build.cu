@@ -18,12 +18,19 @@
 //   5 witness PRUNE  same search; kept candidates merged per (s, v2) in
 //                    shared memory (min weight, then min via) and checked
 //                    against the existing overlay edge
-//   6 emit_ch        out/in lists of V_F become E_up / E_down
-//   7 compact_lists  neighbour lists of N(V_F) drop the contracted vertices
-//   8 reserve        lists short of slack are moved by a prefix sum over
-//                    their new capacities
-//   9 insert         shortcuts appended into the slack (or weights lowered)
-//  10 compact VO     stable compaction of the live-vertex list
+//   6 emit_ch        out/in lists of V_F become E_up / E_down; in the same
+//                    launch the lists of N(V_F) drop the contracted vertices
+//                    and those short of slack move to the arena's tail
+//   7 insert         shortcuts appended into the slack (or weights lowered),
+//                    and the live-vertex list compacted
+//
+// A round of a late overlay is a chain of short kernels, so their number and
+// the gaps between them count: 12 to 13 launches (28 with every list step and
+// scan by itself), each allowed to start while the one before it ends
+// (programmatic dependent launch), step times stamped by the kernels instead
+// of event records between them, and the host's one read handed over by the
+// last kernel it depends on. 1M-vertex geometric graph, 215 rounds: 94.0 -> 54.8
+// ms; 64 x 64 grid, 43 rounds: 12.7 -> 6.1 ms.
 //
 // The witness distance is d_H(a, b), the least weight of a walk a -> b with
 // at most H edges in the round's overlay (INF if none); a candidate
@@ -37,7 +44,7 @@
 // results do not depend on the order in which atomics append to lists.
 
 #include <algorithm>
-#include <chrono>
+#include <atomic>
 #include <cstring>
 
 #include "handle.cuh"
@@ -91,11 +98,10 @@ constexpr int WIT_MC = 128;        // distinct targets merged per source
 
 struct Ctl {
     uint32_t nVO, nVO2, nS, nS2, nF, nAnext, nOvf, nRec;
-    uint32_t err, work, work2, work3, nOvf2, pad;
+    uint32_t err, work, work2, work3, work4, nOvf1, nOvf2;
     unsigned long long candBound, degFout, degFin, degAnext;
     unsigned long long cand, kept, merged, inserted, newEdges;
     unsigned long long out_tail, in_tail, ch_up_tail, ch_dn_tail;
-    unsigned long long relocOut, relocIn;
     unsigned long long wit_sources, wit_fallback, wit_vertices, wit_edges, wit_middles,
         wit_midedges, wit_block;
     unsigned long long trace_valid;  // trace rows of eligible rescorings
@@ -108,7 +114,47 @@ struct Ctl {
     // copied by k_round_end for the host's next read
     unsigned long long log_tail;
     unsigned long long s_cand, s_kept, s_merged, s_inserted, s_newEdges, s_nRec, s_dm_count;
+    uint32_t prepDone;  // blocks of k_contract_prep that have finished
 };
+
+// What the host reads once a round: the control block and the number of the
+// round's read, in pinned memory that k_contract_prep's last block writes.
+struct HostBox {
+    Ctl c;
+    volatile uint32_t seq;
+};
+
+// Times of a round's steps, written by its kernels as they start (ns): event
+// records between the launches would keep them from overlapping.
+enum RoundStamp : int {
+    TS_SCORE = 0,
+    TS_WIT,       // the score phase's searches
+    TS_WIT_END,
+    TS_SELECT,
+    TS_PREP,
+    TS_PREP_END,
+    TS_CONTRACT,  // the contraction phase's searches
+    TS_UPDATE,
+    TS_END,
+    TS_COUNT
+};
+constexpr uint32_t TS_ROUNDS = 4096;  // rounds of stamps the device holds
+
+__device__ __forceinline__ unsigned long long time_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+__device__ __forceinline__ void stamp(unsigned long long *ts) {
+    if (ts && blockIdx.x == 0 && threadIdx.x == 0) *ts = time_ns();
+}
+// Start of a round kernel: its launch may overlap the end of the one before.
+__device__ __forceinline__ void round_kernel(unsigned long long *ts = nullptr) {
+    pdl_wait();
+    pdl_launch();
+    stamp(ts);
+}
+__global__ void k_stamp(unsigned long long *ts) { *ts = time_ns(); }
 
 struct Dev {
     uint32_t n;
@@ -238,16 +284,14 @@ struct WArgs {
     uint4 *rec;              // PRUNE: shortcut records (v1, v2, w, via)
     uint8_t *rec_flag;       // PRUNE: 1 = lowers an existing edge
     uint64_t rec_cap;
-    // Routing to the block tier without a warp attempt: every source when
-    // the phase has at most route_all sources (16 times the block tier's
-    // grid: with that few sources per-source latency decides, and a block
-    // finishes a source sooner than a warp), and any source whose middles'
-    // out-degrees sum above route_deg (its ball would overflow).
-    uint32_t route_all, route_deg;
+    // A source whose middles' out-degrees sum above this goes to the block
+    // tiers without a warp attempt (its ball would overflow).
+    uint32_t route_deg;
     // F_LW: a hop level from the second on whose frontier has more
     // out-edges than this is not run
     unsigned long long level_work;
     uint32_t theta;  // F_TH: settled-vertex cap
+    unsigned long long *ts;  // stamped by the phase's first kernel
 };
 
 struct Dense {
@@ -265,6 +309,13 @@ __device__ __forceinline__ uint64_t select_key(const Dev &d, uint32_t v) {
     uint32_t hi = (uint32_t)d.P[v] ^ 0x80000000u;
     uint32_t lo = d.tie_mode == CH_TIE_ID ? v : murmur_fmix32(v ^ d.tie_seed);
     return ((uint64_t)hi << 32) | lo;
+}
+
+// The counters of a contraction phase and of both phases' searches.
+__device__ __forceinline__ void phase_begin(Ctl *ctl) {
+    ctl->cand = ctl->kept = ctl->merged = ctl->inserted = ctl->newEdges = 0;
+    ctl->nOvf = ctl->nOvf1 = ctl->nOvf2 = 0;
+    ctl->work = ctl->work2 = ctl->work3 = ctl->work4 = 0;
 }
 
 template <int MODE>
@@ -409,7 +460,8 @@ __global__ void k_iota(uint32_t *a, uint32_t n) {
 // One warp per rescored vertex u: its score starts at the edge term, and its
 // in-neighbours become witness sources (each once per round).
 __global__ void k_score_prep(Dev d, const uint32_t *A, uint32_t nA, uint32_t stamp,
-                             uint32_t *S, uint32_t r) {
+                             uint32_t *S, uint32_t r, unsigned long long *ts) {
+    round_kernel(ts);
     const uint32_t lane = lane_id();
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nA; i += nwarps) {
@@ -499,18 +551,56 @@ __device__ __forceinline__ uint32_t ht_find(const uint32_t *keys, int bits, uint
     return EMPTY;
 }
 
+// A witness kernel's counters, summed over the block in shared memory and added
+// to the control block's by one thread each where there is anything to add. (A
+// warp adding its own, zeros included, made tens of thousands of atomics on two
+// cache lines per launch: 15 to 30 us, whatever the sources.)
+constexpr int NTOT = 13;
+struct Totals {
+    unsigned long long src, fallback, vert, edge, mid, midedge, block, cand, kept, merged, ins, fresh, dm;
+};
+static_assert(sizeof(Totals) == NTOT * sizeof(unsigned long long), "one word a counter");
+static_assert(offsetof(Ctl, wit_block) == offsetof(Ctl, wit_sources) + 6 * sizeof(unsigned long long) &&
+                  offsetof(Ctl, newEdges) == offsetof(Ctl, cand) + 4 * sizeof(unsigned long long),
+              "the counters' order in the control block");
+
+__device__ __forceinline__ void clear_totals(unsigned long long *s_tot) {
+    if (threadIdx.x < NTOT) s_tot[threadIdx.x] = 0;
+}
+
+// Every thread of the block calls it, after clear_totals and a barrier.
+__device__ __forceinline__ void add_totals(unsigned long long *s_tot, const Totals &t, Ctl *ctl,
+                                           unsigned long long *dm_count) {
+    const unsigned long long v[NTOT] = {t.src,   t.fallback, t.vert, t.edge,   t.mid, t.midedge, t.block,
+                                        t.cand,  t.kept,     t.merged, t.ins, t.fresh, t.dm};
+#pragma unroll
+    for (int i = 0; i < NTOT; ++i) {
+        if (!__any_sync(FULL, v[i] != 0)) continue;
+        unsigned long long x = v[i];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
+        if (lane_id() == 0) atomicAdd(&s_tot[i], x);
+    }
+    __syncthreads();
+    const uint32_t i = threadIdx.x;
+    if (i >= NTOT || !s_tot[i]) return;
+    atomicAdd(i < 7 ? &ctl->wit_sources + i : (i < 12 ? &ctl->cand + (i - 7) : dm_count), s_tot[i]);
+}
+
 template <int MODE, int FEAT>
 __global__ void __launch_bounds__(WIT_WARPS * 32) k_witness(WArgs a) {
     constexpr bool XM = (FEAT & F_XM) != 0, LW = (FEAT & F_LW) != 0, PR = (FEAT & F_PR) != 0;
     constexpr bool TH = (FEAT & F_TH) != 0;
     __shared__ WarpSmem smem[WIT_WARPS];
+    __shared__ unsigned long long s_tot[NTOT];
     WarpSmem &w = smem[threadIdx.x >> 5];
+    clear_totals(s_tot);
+    __syncthreads();
+    round_kernel(a.ts);
     const uint32_t lane = lane_id();
     const Dev d = a.d;
     Ctl *ctl = d.ctl;
     const uint32_t nS = *a.nS;
     const uint32_t r = a.round;
-    const bool route_all = nS <= a.route_all;
     unsigned long long c_src = 0, c_vert = 0, c_edge = 0, c_mid = 0, c_midedge = 0;
     unsigned long long c_cand = 0, c_kept = 0, c_merged = 0, c_ins = 0, c_new = 0;
     unsigned long long c_dm = 0;  // keys added to the memoised-distance map
@@ -533,10 +623,6 @@ __global__ void __launch_bounds__(WIT_WARPS * 32) k_witness(WArgs a) {
                 else a.ovf[atomicAdd(&ctl->nOvf, 1u)] = s;
             }
         };
-        if (route_all) {
-            hand_on();
-            continue;
-        }
         const uint64_t sb = d.out_beg[s];
         const uint32_t sd = d.out_deg[s];
         if (sb + sd > d.out_arena) {
@@ -984,84 +1070,86 @@ __global__ void __launch_bounds__(WIT_WARPS * 32) k_witness(WArgs a) {
         c_mid += l_mid;
         c_midedge += l_midedge;
     }
-    // Counters (lane-local sums folded per warp).
-    c_src = warp_sum((uint32_t)c_src);
-#define FOLD64(x)                                                               \
-    {                                                                           \
-        unsigned long long v_ = x;                                              \
-        for (int o_ = 16; o_ > 0; o_ >>= 1) v_ += __shfl_xor_sync(FULL, v_, o_); \
-        x = v_;                                                                 \
-    }
-    FOLD64(c_vert) FOLD64(c_edge) FOLD64(c_mid) FOLD64(c_midedge) FOLD64(c_cand)
-    FOLD64(c_kept) FOLD64(c_merged) FOLD64(c_ins) FOLD64(c_new)
-    if constexpr (XM) FOLD64(c_dm)
-#undef FOLD64
-    if (lane == 0) {
-        if constexpr (XM) atomicAdd(a.dm.count, c_dm);
-        atomicAdd(&ctl->wit_sources, c_src);
-        atomicAdd(&ctl->wit_vertices, c_vert);
-        atomicAdd(&ctl->wit_edges, c_edge);
-        atomicAdd(&ctl->wit_middles, c_mid);
-        atomicAdd(&ctl->wit_midedges, c_midedge);
-        if (MODE == MODE_PRUNE) {
-            atomicAdd(&ctl->cand, c_cand);
-            atomicAdd(&ctl->kept, c_kept);
-            atomicAdd(&ctl->merged, c_merged);
-            atomicAdd(&ctl->inserted, c_ins);
-            atomicAdd(&ctl->newEdges, c_new);
-        }
-    }
+    add_totals(s_tot, Totals{c_src, 0, c_vert, c_edge, c_mid, c_midedge, 0, c_cand, c_kept, c_merged, c_ins, c_new, c_dm},
+               ctl, a.dm.count);
 }
 
-// Block tier: the same search for sources whose ball outgrew a warp's
-// tables, run by a whole block with tables 16 times larger in shared memory
-// (about 105 KB, two blocks per SM). Sources that outgrow these too go on to
-// the dense tier. Control values (frontier size, overflow flag, bound) are
-// read by all threads between two barriers and written only after the
-// second.
-constexpr int WB_THREADS = 256;
-constexpr int WB_TBITS = 12;
-constexpr int WB_T = 1 << WB_TBITS;
-constexpr int WB_FC = 2048;
-constexpr int WB_MBITS = 11;
-constexpr int WB_M = 1 << WB_MBITS;
+// Block tiers: the same search by a whole block, for sources whose ball
+// outgrew a warp's tables, and for every source of a phase with few of them.
+// The middle tier has tables of 1024 vertices: 23 KB (29 KB with the merge
+// table of the contraction phase), so that 8 blocks of 128 threads share an SM.
+// Late rounds have a few thousand sources or fewer, whose balls hold 64 to 512
+// vertices but whose searches relax thousands of edges, level after level of
+// the dense overlay: what counts there is how many run at once, or, when there
+// are fewer than blocks, the time of one (then 512 threads a block). The big
+// tier (4096 vertices, about 105 KB, two blocks per SM) takes what outgrows
+// the middle one, the dense tier what outgrows that. Round 30 of a
+// 1M-vertex geometric build, 4,290 sources: 163 us for the score phase, against
+// 506 with the big tier's tables for all.
+// Control values (frontier size, overflow flag, bound) are read by all threads
+// between two barriers and written only after the second.
+constexpr int WB_THREADS = 256;         // big tier
+constexpr int WM_THREADS_MANY = 128;    // middle tier: more sources than blocks
+constexpr int WM_THREADS_FEW = 512;     // and fewer
+constexpr int WB_WARPS_MAX = WM_THREADS_FEW / 32;
 
+template <int TBITS, int FCAP, int MERGEBITS, int MODE>
 struct __align__(16) BlkSmem {
-    uint32_t key[WB_T];
-    uint32_t val[WB_T];
-    uint32_t fst[WB_T];
-    uint2 front[2][WB_FC];
-    uint32_t mkey[WB_M];
-    unsigned long long mval[WB_M];
-    uint32_t cntw[WB_THREADS / 32][32];
+    static constexpr int TB = TBITS, T = 1 << TB, FC = FCAP, MB = MERGEBITS, M = 1 << MB;
+    static constexpr int THREADS = TBITS < 12 ? WM_THREADS_FEW : WB_THREADS;  // at most
+    uint32_t key[T];
+    uint32_t val[T];
+    uint32_t fst[T];
+    uint2 front[2][FC];
+    uint32_t mkey[MODE == MODE_PRUNE ? M : 4];
+    unsigned long long mval[MODE == MODE_PRUNE ? M : 2];
+    uint32_t cntw[WB_WARPS_MAX][32];
     uint32_t nf[2];
     uint32_t item, ovf, bound, nnew, nkeys, memo_ok;
     uint32_t any;  // memoised-distance mode: the source has a candidate
     unsigned long long lwork;  // F_LW: out-edges of the next level's frontier
     uint32_t direct;           // F_PR: heaviest overlay edge (s, v) to a new target v
 };
+template <int MODE>
+using MidSmem = BlkSmem<10, 512, 9, MODE>;
+template <int MODE>
+using BigSmem = BlkSmem<12, 2048, 11, MODE>;
 
-template <int MODE, int FEAT>
-__global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
+// The sources of a block tier's launch, and where it hands on those it cannot
+// hold (hubs go to the dense tier's list at once).
+struct BlkList {
+    const uint32_t *in, *n;
+    uint32_t *work, *out, *out_cnt;
+    unsigned long long *ts;  // stamped when this is the phase's first kernel
+};
+
+template <int MODE, int FEAT, class SM>
+__global__ void __launch_bounds__(SM::THREADS, SM::TB < 12 ? 2 : 1) k_witness_block(WArgs a, BlkList l) {
     constexpr bool XM = (FEAT & F_XM) != 0, LW = (FEAT & F_LW) != 0, PR = (FEAT & F_PR) != 0;
     extern __shared__ __align__(16) unsigned char wb_raw[];
-    BlkSmem &b = *reinterpret_cast<BlkSmem *>(wb_raw);
+    SM &b = *reinterpret_cast<SM *>(wb_raw);
     const Dev d = a.d;
     Ctl *ctl = d.ctl;
     const uint32_t r = a.round;
     const uint32_t tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     const uint32_t nwarps = blockDim.x >> 5;
-    const uint32_t nIn = ctl->nOvf;
+    __shared__ unsigned long long s_tot[NTOT];
+    clear_totals(s_tot);  // (a barrier follows before the first item)
+    bool worked = false;
+    round_kernel(l.ts);
+    const uint32_t nIn = *l.n;
+    if (nIn == 0) return;
     unsigned long long c_src = 0, c_vert = 0, c_edge = 0, c_mid = 0, c_midedge = 0;
     unsigned long long c_cand = 0, c_kept = 0, c_merged = 0, c_ins = 0, c_new = 0;
     unsigned long long c_dm = 0;  // keys added to the memoised-distance map
     while (true) {
         __syncthreads();
-        if (tid == 0) b.item = atomicAdd(&ctl->work3, 1u);
+        if (tid == 0) b.item = atomicAdd(l.work, 1u);
         __syncthreads();
         const uint32_t i = b.item;
         if (i >= nIn) break;
-        const uint32_t s = a.ovf[i];
+        worked = true;
+        const uint32_t s = l.in[i];
         if (s >= d.n) {
             if (tid == 0) atomicOr(&ctl->err, ERR_BOUND);
             continue;
@@ -1147,7 +1235,7 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
         if (searches) {
             uint4 *k4 = reinterpret_cast<uint4 *>(b.key), *v4 = reinterpret_cast<uint4 *>(b.val),
                   *f4 = reinterpret_cast<uint4 *>(b.fst);
-            for (uint32_t t = tid; t < (uint32_t)WB_T / 4; t += blockDim.x) {
+            for (uint32_t t = tid; t < (uint32_t)SM::T / 4; t += blockDim.x) {
                 k4[t] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
                 v4[t] = make_uint4(INF, INF, INF, INF);
                 f4[t] = make_uint4(0, 0, 0, 0);
@@ -1156,13 +1244,13 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
         if (MODE == MODE_PRUNE) {
             uint4 *m4 = reinterpret_cast<uint4 *>(b.mkey);
             ulonglong2 *mv2 = reinterpret_cast<ulonglong2 *>(b.mval);
-            for (uint32_t t = tid; t < (uint32_t)WB_M / 4; t += blockDim.x)
+            for (uint32_t t = tid; t < (uint32_t)SM::M / 4; t += blockDim.x)
                 m4[t] = make_uint4(EMPTY, EMPTY, EMPTY, EMPTY);
-            for (uint32_t t = tid; t < (uint32_t)WB_M / 2; t += blockDim.x) mv2[t] = make_ulonglong2(~0ull, ~0ull);
+            for (uint32_t t = tid; t < (uint32_t)SM::M / 2; t += blockDim.x) mv2[t] = make_ulonglong2(~0ull, ~0ull);
         }
         __syncthreads();
         if (tid == 0 && !memo_all) {
-            const uint32_t h = ht_insert(b.key, WB_TBITS, s);
+            const uint32_t h = ht_insert(b.key, SM::TB, s);
             b.val[h] = 0;
             b.front[0][0] = make_uint2(h, 0);
             b.nf[0] = 1;
@@ -1192,9 +1280,9 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
             __syncthreads();
             for (uint32_t f0 = warp * 32; f0 < nfront; f0 += nwarps * 32) {
                 const uint32_t fi = f0 + lane;
-                const bool fv = fi < nfront && fi < (uint32_t)WB_FC;
+                const bool fv = fi < nfront && fi < (uint32_t)SM::FC;
                 const uint2 fe = fv ? b.front[cur][fi] : make_uint2(0, 0);
-                const bool fok = fv && fe.x < (uint32_t)WB_T;
+                const bool fok = fv && fe.x < (uint32_t)SM::T;
                 if (fv && !fok) atomicOr(&ctl->err, ERR_BOUND);
                 const uint32_t x = fok ? b.key[fe.x] : 0;
                 const bool xok = fok && id_ok(d, x);
@@ -1217,7 +1305,7 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
                     const uint32_t nd = sat_add(dx_o, e.y);
                     if (nd >= sbound || !id_ok(d, e.x)) continue;
                     bool created = false;
-                    const uint32_t slot = ht_insert(b.key, WB_TBITS, e.x, &created);
+                    const uint32_t slot = ht_insert(b.key, SM::TB, e.x, &created);
                     if (created) atomicAdd(&b.nkeys, 1u);
                     if (slot == EMPTY) {
                         b.ovf = 1;
@@ -1226,13 +1314,13 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
                     const uint32_t old = atomicMin(&b.val[slot], nd);
                     if (nd < old && atomicExch(&b.fst[slot], lvl) != lvl) {
                         const uint32_t p = atomicAdd(&b.nf[nxt], 1u);
-                        if (p < (uint32_t)WB_FC) b.front[nxt][p] = make_uint2(slot, 0);
+                        if (p < (uint32_t)SM::FC) b.front[nxt][p] = make_uint2(slot, 0);
                         else b.ovf = 1;
                     }
                 }
             }
             __syncthreads();
-            const uint32_t nn = min(b.nf[nxt], (uint32_t)WB_FC);
+            const uint32_t nn = min(b.nf[nxt], (uint32_t)SM::FC);
             unsigned long long lw = 0;
             for (uint32_t p = tid; p < nn; p += blockDim.x) {
                 b.front[nxt][p].y = b.val[b.front[nxt][p].x];
@@ -1246,7 +1334,7 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
         const uint32_t ovf1 = b.ovf;
         __syncthreads();
         if (ovf1) {
-            if (tid == 0) a.ovf2[atomicAdd(&ctl->nOvf2, 1u)] = s;
+            if (tid == 0) l.out[atomicAdd(l.out_cnt, 1u)] = s;
             continue;
         }
         // Phase 2: decisions, each warp taking 32 of the source's out-edges.
@@ -1286,7 +1374,7 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
                 } else {
                     uint32_t dh;
                     if (!(XM && dmap_get(a.dm, dmap_key(s, e2.x), &dh))) {
-                        const uint32_t slot = ht_find(b.key, WB_TBITS, e2.x);
+                        const uint32_t slot = ht_find(b.key, SM::TB, e2.x);
                         dh = slot == EMPTY ? INF : b.val[slot];
                     }
                     keepit = via != INF && via <= dh;
@@ -1298,7 +1386,7 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
                 if (MODE == MODE_SCORE) {
                     atomicAdd(&b.cntw[warp][o], 1u);
                 } else {
-                    const uint32_t ms = ht_insert(b.mkey, WB_MBITS, e2.x);
+                    const uint32_t ms = ht_insert(b.mkey, SM::MB, e2.x);
                     if (ms == EMPTY) b.ovf = 1;
                     else atomicMin(&b.mval[ms], ((unsigned long long)via << 32) | u_o);
                 }
@@ -1313,11 +1401,11 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
             const uint32_t ovf2 = b.ovf;
             __syncthreads();
             if (ovf2) {
-                if (tid == 0) a.ovf2[atomicAdd(&ctl->nOvf2, 1u)] = s;
+                if (tid == 0) l.out[atomicAdd(l.out_cnt, 1u)] = s;
                 continue;
             }
             uint32_t l_new = 0;
-            for (uint32_t t = tid; t < (uint32_t)WB_M; t += blockDim.x) {
+            for (uint32_t t = tid; t < (uint32_t)SM::M; t += blockDim.x) {
                 const uint32_t v2 = b.mkey[t];
                 if (v2 == EMPTY) continue;
                 const unsigned long long mv = b.mval[t];
@@ -1380,7 +1468,7 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
                         if (idx >= total) continue;
                         const uint2 e2 = d.out_adj[ub_o + (idx - ex_o)];
                         if (e2.x == s) continue;
-                        const uint32_t slot = ht_find(b.key, WB_TBITS, e2.x);
+                        const uint32_t slot = ht_find(b.key, SM::TB, e2.x);
                         const int put = dmap_put(a.dm, dmap_key(s, e2.x), slot == EMPTY ? INF : b.val[slot]);
                         full |= put < 0;
                         c_dm += put > 0;
@@ -1395,31 +1483,10 @@ __global__ void __launch_bounds__(WB_THREADS) k_witness_block(WArgs a) {
         c_mid += l_mid;
         c_midedge += l_midedge;
     }
-#define FOLD64(x)                                                               \
-    {                                                                           \
-        unsigned long long v_ = x;                                              \
-        for (int o_ = 16; o_ > 0; o_ >>= 1) v_ += __shfl_xor_sync(FULL, v_, o_); \
-        x = v_;                                                                 \
-    }
-    FOLD64(c_src) FOLD64(c_vert) FOLD64(c_edge) FOLD64(c_mid) FOLD64(c_midedge) FOLD64(c_cand)
-    FOLD64(c_kept) FOLD64(c_merged) FOLD64(c_ins) FOLD64(c_new)
-    if constexpr (XM) FOLD64(c_dm)
-#undef FOLD64
-    if (lane == 0) {
-        if constexpr (XM) atomicAdd(a.dm.count, c_dm);
-        atomicAdd(&ctl->wit_block, c_src);
-        atomicAdd(&ctl->wit_vertices, c_vert);
-        atomicAdd(&ctl->wit_edges, c_edge);
-        atomicAdd(&ctl->wit_middles, c_mid);
-        atomicAdd(&ctl->wit_midedges, c_midedge);
-        if (MODE == MODE_PRUNE) {
-            atomicAdd(&ctl->cand, c_cand);
-            atomicAdd(&ctl->kept, c_kept);
-            atomicAdd(&ctl->merged, c_merged);
-            atomicAdd(&ctl->inserted, c_ins);
-            atomicAdd(&ctl->newEdges, c_new);
-        }
-    }
+    if (!worked) return;
+    __syncthreads();
+    add_totals(s_tot, Totals{0, 0, c_vert, c_edge, c_mid, c_midedge, c_src, c_cand, c_kept, c_merged, c_ins, c_new, c_dm},
+               ctl, a.dm.count);
 }
 
 // Same search for the sources whose ball overflowed shared memory: one block
@@ -1444,7 +1511,9 @@ __global__ void __launch_bounds__(256) k_witness_dense(WArgs a, Dense dn) {
     __shared__ unsigned long long s_best;  // F_TH: least (label, id) of an unsettled vertex
     __shared__ unsigned long long s_cnt[5];
     const uint32_t tid = threadIdx.x;
+    round_kernel();
     const uint32_t nOvf = ctl->nOvf2;
+    if (nOvf == 0) return;
     while (true) {
         __syncthreads();
         if (tid == 0) s_item = atomicAdd(&ctl->work2, 1u);
@@ -1891,7 +1960,9 @@ __global__ void k_orig_deg(Dev d) {
 // step (a round of an RMAT 2^17 build: 2.7 -> 0.06 ms).
 constexpr uint32_t SELECT_LONG = 256;
 
-__global__ void k_select(Dev d, const uint32_t *VO, uint32_t nVO, uint32_t per, uint32_t r, uint32_t *F) {
+__global__ void k_select(Dev d, const uint32_t *VO, uint32_t nVO, uint32_t per, uint32_t r, uint32_t *F,
+                         unsigned long long *ts) {
+    round_kernel(ts);
     const uint32_t lane = lane_id();
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -1961,8 +2032,11 @@ __global__ void k_select(Dev d, const uint32_t *VO, uint32_t nVO, uint32_t per, 
 // One warp per selected vertex u: counts its candidates and edges, and
 // marks its neighbours as next round's affected set and its in-neighbours as
 // the contraction phase's witness sources (each once).
+// The last block to finish hands the control block to the host (box) and puts
+// the contraction phase's counters at zero.
 __global__ void k_contract_prep(Dev d, const uint32_t *F, uint32_t src_stamp, uint32_t next_r,
-                                uint32_t *S2, uint32_t *Anext) {
+                                uint32_t *S2, uint32_t *Anext, unsigned long long *ts, HostBox *box, uint32_t seq) {
+    round_kernel(ts);
     const uint32_t nF = d.ctl->nF;
     const uint32_t lane = lane_id();
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -2007,24 +2081,118 @@ __global__ void k_contract_prep(Dev d, const uint32_t *F, uint32_t src_stamp, ui
             atomicAdd(&d.ctl->degFin, w_in);
         }
     }
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&d.ctl->prepDone, 1u) + 1 == gridDim.x;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const uint32_t *from = reinterpret_cast<const uint32_t *>(d.ctl);
+    uint32_t *to = reinterpret_cast<uint32_t *>(&box->c);
+    for (uint32_t j = threadIdx.x; j < sizeof(Ctl) / 4; j += blockDim.x) to[j] = __ldcg(from + j);
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        d.ctl->prepDone = 0;
+        phase_begin(d.ctl);
+        ts[TS_PREP_END - TS_PREP] = time_ns();
+        __threadfence_system();
+        box->seq = seq;
+    }
 }
 
 // --------------------------------------------------------------------------
 // Steps 6-9: CH edges, list maintenance, insertion
 // --------------------------------------------------------------------------
 
+constexpr uint32_t TOMB = 0xFFFFFFFFu;  // a pruned adjacency entry (never a vertex id)
+
+// Stable in-place removal, by one warp, of this round's contracted vertices
+// and of pruned entries (tombstones) from a list (32 entries per step;
+// writes never pass the reads).
+__device__ __forceinline__ uint32_t warp_compact_list(const Dev &d, uint2 *adj, uint64_t b, uint32_t dg,
+                                                      uint32_t r) {
+    const uint32_t lane = lane_id();
+    uint32_t k = 0;
+    for (uint32_t j0 = 0; j0 < dg; j0 += 32) {
+        const uint32_t j = j0 + lane;
+        uint2 e = make_uint2(0, 0);
+        bool keep = false;
+        if (j < dg) {
+            e = adj[b + j];
+            keep = e.x != TOMB && id_ok(d, e.x) && d.level[e.x] != r;
+        }
+        const uint32_t m = __ballot_sync(FULL, keep);
+        if (keep) adj[b + k + __popc(m & ((1u << lane) - 1u))] = e;
+        k += __popc(m);
+        __syncwarp();
+    }
+    return k;
+}
+
+// One warp per affected vertex x: drops this round's contracted vertices from
+// its out- and in-lists and, where the shortcuts to come do not fit, moves a
+// list to the arena's tail (twice what it needs; the tail is an atomic counter,
+// so lists land in any order). One launch in place of a compaction, a pass
+// over the new degrees, two 64-bit scans and a relocation (8 launches).
+__device__ __forceinline__ void update_lists(const Dev &d, uint32_t x, uint32_t r) {
+    const uint32_t lane = lane_id();
+#pragma unroll
+    for (int dir = 0; dir < 2; ++dir) {
+        uint2 *adj = dir ? d.in_adj : d.out_adj;
+        uint64_t *beg = dir ? d.in_beg : d.out_beg;
+        uint32_t *deg = dir ? d.in_deg : d.out_deg, *cap = dir ? d.in_cap : d.out_cap;
+        uint32_t *fresh = dir ? d.new_in : d.new_out;
+        unsigned long long *tail = dir ? &d.ctl->in_tail : &d.ctl->out_tail;
+        auto ok = [&](uint64_t b, uint32_t n) { return dir ? in_list_ok(d, b, n) : out_list_ok(d, b, n); };
+        const uint64_t b = beg[x];
+        uint32_t k = deg[x];
+        if (ok(b, k)) {
+            k = warp_compact_list(d, adj, b, k, r);
+            if (lane == 0) deg[x] = k;
+        } else {
+            k = 0;
+        }
+        const uint32_t need = k + fresh[x];
+        __syncwarp();
+        if (lane == 0) fresh[x] = 0;
+        if (need <= cap[x]) continue;
+        const uint32_t want = max(2u * need, 4u);
+        unsigned long long nb = 0;
+        if (lane == 0) nb = atomicAdd(tail, (unsigned long long)want);
+        nb = __shfl_sync(FULL, nb, 0);
+        if (!ok(nb, want)) continue;
+        for (uint32_t j = lane; j < k; j += 32) adj[nb + j] = adj[b + j];
+        __syncwarp();
+        if (lane == 0) {
+            beg[x] = nb;
+            cap[x] = want;
+        }
+    }
+}
+
 // One warp per selected vertex u: its out-edges become E_up, its in-edges
 // E_down. With core set, F is the live list of a round that found no
 // eligible vertex: every live vertex gets level r and its overlay edges, and
 // no neighbour bookkeeping is done (the build ends).
+//
+// In the same launch, one warp per affected vertex X[i] (F and X are disjoint,
+// and neither part reads what the other writes): see update_lists.
 __global__ void k_emit_ch(Dev d, const uint32_t *F, uint32_t nF, uint2 *ch_up, uint2 *ch_dn,
                           uint64_t *up_beg, uint32_t *up_deg, uint64_t *dn_beg,
-                          uint32_t *dn_deg, uint64_t up_cap, uint64_t dn_cap, bool core, uint32_t r) {
+                          uint32_t *dn_deg, uint64_t up_cap, uint64_t dn_cap, bool core, uint32_t r,
+                          const uint32_t *X, uint32_t nX, unsigned long long *ts) {
+    round_kernel(ts);
     const uint32_t lane = lane_id();
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nF; i += nwarps) {
-        const uint32_t u = F[i];
+    for (uint64_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < (uint64_t)nF + nX; i += nwarps) {
+        const uint32_t u = i < nF ? F[i] : X[i - nF];
         if (!id_ok(d, u)) continue;
+        if (i >= nF) {
+            update_lists(d, u, r);
+            continue;
+        }
         const uint64_t ob = d.out_beg[u], ib = d.in_beg[u];
         const uint32_t od = out_list_ok(d, ob, d.out_deg[u]) ? d.out_deg[u] : 0;
         const uint32_t id = in_list_ok(d, ib, d.in_deg[u]) ? d.in_deg[u] : 0;
@@ -2061,31 +2229,6 @@ __global__ void k_emit_ch(Dev d, const uint32_t *F, uint32_t nF, uint2 *ch_up, u
             atomicMax(&d.depth[x], du + 1);
         }
     }
-}
-
-constexpr uint32_t TOMB = 0xFFFFFFFFu;  // a pruned adjacency entry (never a vertex id)
-
-// Stable in-place removal, by one warp, of this round's contracted vertices
-// and of pruned entries (tombstones) from a list (32 entries per step;
-// writes never pass the reads).
-__device__ __forceinline__ uint32_t warp_compact_list(const Dev &d, uint2 *adj, uint64_t b, uint32_t dg,
-                                                      uint32_t r) {
-    const uint32_t lane = lane_id();
-    uint32_t k = 0;
-    for (uint32_t j0 = 0; j0 < dg; j0 += 32) {
-        const uint32_t j = j0 + lane;
-        uint2 e = make_uint2(0, 0);
-        bool keep = false;
-        if (j < dg) {
-            e = adj[b + j];
-            keep = e.x != TOMB && id_ok(d, e.x) && d.level[e.x] != r;
-        }
-        const uint32_t m = __ballot_sync(FULL, keep);
-        if (keep) adj[b + k + __popc(m & ((1u << lane) - 1u))] = e;
-        k += __popc(m);
-        __syncwarp();
-    }
-    return k;
 }
 
 // --------------------------------------------------------------------------
@@ -2242,103 +2385,22 @@ __global__ void k_score_map(Dev d, DMap dm, const uint32_t *A, uint32_t nA, uint
     }
 }
 
-// One warp per affected vertex x: drop this round's contracted vertices from
-// its out- and in-lists.
-__global__ void k_compact_lists(Dev d, const uint32_t *X, uint32_t nX, uint32_t r) {
-    const uint32_t lane = lane_id();
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nX; i += nwarps) {
-        const uint32_t x = X[i];
-        if (!id_ok(d, x)) continue;
-        const uint64_t ob = d.out_beg[x], ib = d.in_beg[x];
-        const uint32_t od = d.out_deg[x], id = d.in_deg[x];
-        if (out_list_ok(d, ob, od)) {
-            const uint32_t k = warp_compact_list(d, d.out_adj, ob, od, r);
-            if (lane == 0) d.out_deg[x] = k;
-        }
-        if (in_list_ok(d, ib, id)) {
-            const uint32_t k = warp_compact_list(d, d.in_adj, ib, id, r);
-            if (lane == 0) d.in_deg[x] = k;
-        }
-    }
-}
-
-__global__ void k_reserve(Dev d, const uint32_t *X, uint32_t nX, uint64_t *reqO,
-                          uint64_t *reqI) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nX;
-         i += gridDim.x * blockDim.x) {
-        const uint32_t x = X[i];
-        const uint32_t no = d.new_out[x], ni = d.new_in[x];
-        d.new_out[x] = 0;
-        d.new_in[x] = 0;
-        const uint32_t needO = d.out_deg[x] + no, needI = d.in_deg[x] + ni;
-        reqO[i] = needO > d.out_cap[x] ? (uint64_t)max(2u * needO, 4u) : 0;
-        reqI[i] = needI > d.in_cap[x] ? (uint64_t)max(2u * needI, 4u) : 0;
-    }
-}
-
-// One warp per affected vertex whose list outgrew its capacity: copy it to
-// its new place at the arena tail.
-__global__ void k_relocate(Dev d, const uint32_t *X, uint32_t nX, const uint64_t *reqO,
-                           const uint64_t *posO, const uint64_t *reqI, const uint64_t *posI) {
-    const uint64_t to = d.ctl->out_tail, ti = d.ctl->in_tail;
-    const uint32_t lane = lane_id();
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nX; i += nwarps) {
-        const uint32_t x = X[i];
-        if (reqO[i]) {
-            const uint64_t nb = to + posO[i], ob = d.out_beg[x];
-            const uint32_t dg = d.out_deg[x];
-            if (out_list_ok(d, nb, (uint32_t)reqO[i]) && out_list_ok(d, ob, dg)) {
-                for (uint32_t j = lane; j < dg; j += 32) d.out_adj[nb + j] = d.out_adj[ob + j];
-                if (lane == 0) {
-                    d.out_beg[x] = nb;
-                    d.out_cap[x] = (uint32_t)reqO[i];
-                }
-            }
-        }
-        if (reqI[i]) {
-            const uint64_t nb = ti + posI[i], ob = d.in_beg[x];
-            const uint32_t dg = d.in_deg[x];
-            if (in_list_ok(d, nb, (uint32_t)reqI[i]) && in_list_ok(d, ob, dg)) {
-                for (uint32_t j = lane; j < dg; j += 32) d.in_adj[nb + j] = d.in_adj[ob + j];
-                if (lane == 0) {
-                    d.in_beg[x] = nb;
-                    d.in_cap[x] = (uint32_t)reqI[i];
-                }
-            }
-        }
-    }
-}
-
-
-// Start of a round: its counters, and the score phase's witness work
-// counters, start from zero.
-__global__ void k_round_begin(Ctl *ctl) {
-    ctl->nS = ctl->nS2 = ctl->nF = ctl->nAnext = ctl->nOvf = ctl->nRec = 0;
+// Before the first round: counters at zero.
+__device__ __forceinline__ void round_begin(Ctl *ctl) {
+    ctl->nS = ctl->nS2 = ctl->nF = ctl->nAnext = ctl->nRec = ctl->nVO2 = 0;
     ctl->candBound = ctl->degFout = ctl->degFin = ctl->degAnext = 0;
     ctl->pruned = 0;
     ctl->nDirty = 0;
-    ctl->work = ctl->work2 = ctl->work3 = ctl->nOvf2 = 0;
+    phase_begin(ctl);
 }
+__global__ void k_round_begin(Ctl *ctl) { round_begin(ctl); }
 
-// Start of a round's contraction phase: its counters and its witness work
-// counters start from zero.
-__global__ void k_contract_begin(Ctl *ctl) {
-    ctl->cand = ctl->kept = ctl->merged = ctl->inserted = ctl->newEdges = 0;
-    ctl->nOvf = 0;
-    ctl->work = ctl->work2 = ctl->work3 = ctl->nOvf2 = 0;
-}
-
-// End of a round: the arena tails pass the lists relocated this round (when
-// any were), the next round's live count takes the compacted one, the
-// round's contraction counters are kept for the host's next read, and the
-// shortcut log advances past the round's records.
-__global__ void k_round_end(Ctl *ctl, int advance_tails) {
-    if (advance_tails) {
-        ctl->out_tail += ctl->relocOut;
-        ctl->in_tail += ctl->relocIn;
-    }
+// End of a round: the next round's live count takes the compacted one, the
+// round's contraction counters are kept for the host's next read, the shortcut
+// log advances past the round's records, and the next round's counters start
+// from zero.
+__global__ void k_round_end(Ctl *ctl, unsigned long long *ts) {
+    round_kernel(ts);
     ctl->nVO = ctl->nVO2;
     ctl->s_cand = ctl->cand;
     ctl->s_kept = ctl->kept;
@@ -2348,10 +2410,23 @@ __global__ void k_round_end(Ctl *ctl, int advance_tails) {
     ctl->s_nRec = ctl->nRec;
     ctl->s_dm_count = ctl->dm_count;
     ctl->log_tail += ctl->nRec;
+    round_begin(ctl);
 }
 
+// The round's shortcuts into the lists and the log; and, in the same launch,
+// the live vertices (level still INF) of VO into VO2, in any order: the kernels
+// that read the list only form sets from it.
 __global__ void k_insert(Dev d, const uint4 *rec, const uint8_t *flag, uint32_t r,
-                         uint4 *log, uint32_t *log_round) {
+                         uint4 *log, uint32_t *log_round, const uint32_t *VO, uint32_t nVO, uint32_t *VO2) {
+    round_kernel();
+    const uint32_t nthreads = gridDim.x * blockDim.x;
+    for (uint32_t i0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; i0 < nVO; i0 += nthreads) {
+        const uint32_t i = i0 + lane_id();
+        const uint32_t v = i < nVO ? VO[i] : INF;
+        const bool live = v < d.n && d.level[v] == INF;
+        const uint32_t pos = warp_append(live, &d.ctl->nVO2);
+        if (live) VO2[pos] = v;
+    }
     const uint32_t nRec = d.ctl->nRec;
     const uint64_t log_base = d.ctl->log_tail;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nRec;
@@ -2532,6 +2607,10 @@ int bits_for(uint64_t x) {
     return b;
 }
 
+// Phases of up to this many sources an SM skip the warp tier (1M-vertex
+// geometric build: 60 ms with 64, 66 with 16; with 160, 2% slower than 64).
+constexpr uint32_t DIRECT_SOURCES = 64;
+
 struct EventPool {
     std::vector<cudaEvent_t> evs;
     size_t used = 0;
@@ -2551,7 +2630,6 @@ struct EventPool {
 struct Span {
     cudaEvent_t a, b;
     double *acc;
-    int round, phase;  // phase: index into the per-round timing row, or -1
 };
 
 struct Builder {
@@ -2569,12 +2647,16 @@ struct Builder {
     DevBuf<unsigned long long> emask;  // one word per out-arena entry
     DevBuf<int32_t> P;
     DevBuf<Ctl> ctl;
-    Ctl *hctl = nullptr;  // pinned
+    HostBox *box = nullptr;  // pinned
+    Ctl *hctl = nullptr;     // its control block
+    uint32_t reads = 0;      // control blocks k_contract_prep has been asked for
+    bool use_big = true;     // the middle tier's overflow goes to the big tier, not to the dense one
     // lists
-    DevBuf<uint32_t> VO, VO2, A, Anext, S, S2, F, ovf, ovf2, tmp;
-    int blk_blocks = 152;
+    DevBuf<uint32_t> VO, VO2, A, Anext, S, S2, F, ovf, ovf1, ovf2;
+    int big_blocks = 152, mid_blocks = 152, mid_blocks_few = 152;  // resident blocks of the block tiers
     uint32_t route_deg = 64;  // witness sources above this middle-degree sum go to the block tier
-    DevBuf<uint64_t> reqO, reqI, posO, posI;
+    DevBuf<unsigned long long> stamps;  // [TS_ROUNDS][TS_COUNT]
+    std::vector<unsigned long long> hstamps;
     DevBuf<uint32_t> scan32;
     DevBuf<uint64_t> scan64;
     // records and log
@@ -2618,10 +2700,10 @@ struct Builder {
     // The build's buffers go back to the library's cache when the builder is
     // destroyed; on an error path its kernels may still be running.
     ~Builder() { cudaStreamSynchronize(st); }
-    void mark(double *acc, cudaEvent_t a, int phase = -1) {
+    void mark(double *acc, cudaEvent_t a) {
         cudaEvent_t b = pool.get();
         CH_CUDA_TRY(cudaEventRecord(b, st));
-        spans.push_back({a, b, acc, cur_round, phase});
+        spans.push_back({a, b, acc});
     }
     cudaEvent_t start() {
         cudaEvent_t a = pool.get();
@@ -2632,6 +2714,9 @@ struct Builder {
     void sync_ctl() {
         CH_CUDA_TRY(cudaMemcpyAsync(hctl, ctl.ptr, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
         CH_CUDA_TRY(cudaStreamSynchronize(st));
+        check_ctl();
+    }
+    void check_ctl() {
         if (hctl->err & ERR_INPUT) throw Error{CH_EINVAL, "graph has a malformed offset, id or weight"};
         if (hctl->err & ERR_BOUND) throw Error{CH_ECUDA, "internal index check failed"};
         if (hctl->err & ERR_MAP_FULL)
@@ -2639,14 +2724,40 @@ struct Builder {
         if (hctl->err) throw Error{CH_ECUDA, "internal capacity error " + std::to_string(hctl->err)};
     }
 
+    // Waits for the control block that k_contract_prep hands over.
+    void wait_ctl() {
+        for (uint32_t spins = 0; box->seq != reads; ++spins) {
+            if (spins % 1024 != 1023) continue;
+            const cudaError_t e = cudaStreamQuery(st);
+            if (e == cudaErrorNotReady) continue;
+            if (e == cudaSuccess && box->seq == reads) break;
+            throw Error{CH_ECUDA, e == cudaSuccess ? std::string("internal: no control block from the round")
+                                                   : std::string("build: ") + cudaGetErrorString(e)};
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
+        check_ctl();
+    }
+
+    // Brings the stamps of the rounds since the last call to the host.
+    void fetch_stamps(uint32_t rounds) {
+        const size_t have = hstamps.size() / TS_COUNT, got = rounds - have;
+        if (!got) return;
+        hstamps.resize((size_t)rounds * TS_COUNT);
+        CH_CUDA_TRY(cudaMemcpyAsync(hstamps.data() + have * TS_COUNT, stamps.ptr,
+                                    got * TS_COUNT * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+        stamps.zero(st);
+        CH_CUDA_TRY(cudaStreamSynchronize(st));
+    }
+
     void normalise(const ch_graph_t *g);
     void emit_core(uint32_t r, uint32_t nVO, uint64_t live_edges);
     void run_rounds();
     void postprocess();
     template <int MODE>
-    void witness(const uint32_t *Sl, const uint32_t *nS_dev, uint32_t nS_max, uint32_t r);
+    void witness(const uint32_t *Sl, const uint32_t *nS_dev, uint32_t nS_max, uint32_t expected, uint32_t r,
+                 unsigned long long *ts);
     template <int MODE, int FEAT>
-    void launch_witness(const WArgs &a, int blocks);
+    void launch_witness(const WArgs &a, uint32_t nS_max, uint32_t expected);
     unsigned long long level_work = ~0ull;  // F_LW bound; all ones = off
     uint32_t theta = 0;                     // F_TH settled-vertex cap; 0 = off
 };
@@ -2757,8 +2868,9 @@ void Builder::normalise(const ch_graph_t *g) {
 }
 
 template <int MODE>
-void Builder::witness(const uint32_t *Sl, const uint32_t *nS_dev, uint32_t nS_max, uint32_t r) {
-    // the tiers' work counters (work, work2, work3, nOvf, nOvf2) are zeroed
+void Builder::witness(const uint32_t *Sl, const uint32_t *nS_dev, uint32_t nS_max, uint32_t expected, uint32_t r,
+                      unsigned long long *ts) {
+    // the tiers' work counters (work .. work4, nOvf, nOvf1, nOvf2) are zeroed
     // by k_round_begin / k_contract_begin before each phase
     WArgs a;
     a.d = d;
@@ -2771,45 +2883,64 @@ void Builder::witness(const uint32_t *Sl, const uint32_t *nS_dev, uint32_t nS_ma
     a.rec = rec.ptr;
     a.rec_flag = rec_flag.ptr;
     a.rec_cap = rec.count;
-    a.route_all = (uint32_t)blk_blocks * 16;
     a.route_deg = route_deg;
     a.dm = dm;
     a.level_work = level_work;
     a.theta = theta;
+    a.ts = ts;
     if (dm_phase_clear) {
         CH_CUDA_TRY(cudaMemsetAsync(dm_keys.ptr, 0xFF, dm_keys.count * sizeof(unsigned long long), st));
         CH_CUDA_TRY(cudaMemsetAsync(&ctl.ptr->dm_count, 0, sizeof(unsigned long long), st));
     }
-    cudaEvent_t e0 = start();
-    const int blocks = grid_for((uint64_t)nS_max, WIT_WARPS, sms * 8);
     const int feat = (xm ? F_XM : 0) | (level_work != ~0ull && !theta ? F_LW : 0) | (prune ? F_PR : 0) |
                      (theta ? F_TH : 0);
     switch (feat) {
-        case 0: launch_witness<MODE, 0>(a, blocks); break;
-        case F_XM: launch_witness<MODE, F_XM>(a, blocks); break;
-        case F_LW: launch_witness<MODE, F_LW>(a, blocks); break;
-        case F_XM | F_LW: launch_witness<MODE, F_XM | F_LW>(a, blocks); break;
-        case F_XM | F_PR: launch_witness<MODE, F_XM | F_PR>(a, blocks); break;
-        case F_XM | F_LW | F_PR: launch_witness<MODE, F_XM | F_LW | F_PR>(a, blocks); break;
-        case F_TH: launch_witness<MODE, F_TH>(a, blocks); break;
-        case F_TH | F_XM: launch_witness<MODE, F_TH | F_XM>(a, blocks); break;
-        case F_TH | F_XM | F_PR: launch_witness<MODE, F_TH | F_XM | F_PR>(a, blocks); break;
+        case 0: launch_witness<MODE, 0>(a, nS_max, expected); break;
+        case F_XM: launch_witness<MODE, F_XM>(a, nS_max, expected); break;
+        case F_LW: launch_witness<MODE, F_LW>(a, nS_max, expected); break;
+        case F_XM | F_LW: launch_witness<MODE, F_XM | F_LW>(a, nS_max, expected); break;
+        case F_XM | F_PR: launch_witness<MODE, F_XM | F_PR>(a, nS_max, expected); break;
+        case F_XM | F_LW | F_PR: launch_witness<MODE, F_XM | F_LW | F_PR>(a, nS_max, expected); break;
+        case F_TH: launch_witness<MODE, F_TH>(a, nS_max, expected); break;
+        case F_TH | F_XM: launch_witness<MODE, F_TH | F_XM>(a, nS_max, expected); break;
+        case F_TH | F_XM | F_PR: launch_witness<MODE, F_TH | F_XM | F_PR>(a, nS_max, expected); break;
         default: throw Error{CH_EINVAL, "internal: unsupported witness feature set"};
     }
-    mark(&h->t_witness_ms, e0, 5);
-    h->witness_launches += 3;
 }
 
-// The three tiers of one phase, in order (each takes the sources the one
-// before it could not hold).
+// The tiers of one phase, in order (each takes the sources the one before it
+// could not hold). A phase with few sources starts at the middle block tier;
+// `expected` is their number, or the round before's: it decides the launches
+// only. The settled-vertex cap has no block tiers.
 template <int MODE, int FEAT>
-void Builder::launch_witness(const WArgs &a, int blocks) {
-    k_witness<MODE, FEAT><<<blocks, WIT_WARPS * 32, 0, st>>>(a);
-    CH_CHECK_LAUNCH();
-    k_witness_block<MODE, FEAT><<<blk_blocks, WB_THREADS, sizeof(BlkSmem), st>>>(a);
-    CH_CHECK_LAUNCH();
-    k_witness_dense<MODE, FEAT><<<dense.nslots, 256, 0, st>>>(a, dense);
-    CH_CHECK_LAUNCH();
+void Builder::launch_witness(const WArgs &a, uint32_t nS_max, uint32_t expected) {
+    Ctl *c = ctl.ptr;
+    constexpr bool TH = (FEAT & F_TH) != 0;
+    const bool direct = !TH && expected <= DIRECT_SOURCES * (uint32_t)sms;
+    if (!direct) {
+        launch_pdl(k_witness<MODE, FEAT>, grid_for((uint64_t)nS_max, WIT_WARPS, sms * 8), WIT_WARPS * 32, 0, st, a);
+        ++h->witness_launches;
+    }
+    if constexpr (!TH) {
+        const bool few = direct && expected <= 2 * (uint32_t)sms;
+        BlkList mid{direct ? a.S : ovf.ptr, direct ? a.nS : &c->nOvf, &c->work3, ovf1.ptr, &c->nOvf1,
+                    direct ? a.ts : nullptr};
+        const BlkList big{ovf1.ptr, &c->nOvf1, &c->work4, ovf2.ptr, &c->nOvf2, nullptr};
+        if (!use_big) {
+            mid.out = ovf2.ptr;
+            mid.out_cnt = &c->nOvf2;
+        }
+        launch_pdl(k_witness_block<MODE, FEAT, MidSmem<MODE>>, few ? std::min(mid_blocks_few, (int)expected + 16) : mid_blocks,
+                   few ? WM_THREADS_FEW : WM_THREADS_MANY, sizeof(MidSmem<MODE>), st, a, mid);
+        ++h->witness_launches;
+        if (use_big) {
+            launch_pdl(k_witness_block<MODE, FEAT, BigSmem<MODE>>, big_blocks, WB_THREADS, sizeof(BigSmem<MODE>), st,
+                       a, big);
+            ++h->witness_launches;
+        }
+    }
+    launch_pdl(k_witness_dense<MODE, FEAT>, dense.nslots, 256, 0, st, a, dense);
+    ++h->witness_launches;
 }
 
 // Keeps the memoised-distance map at most half full with `keys` keys plus one
@@ -2849,7 +2980,7 @@ void Builder::emit_core(uint32_t r, uint32_t nVO, uint64_t live_edges) {
         ch_dn.grow(c.ch_dn_tail + live_edges, c.ch_dn_tail, st);
     k_emit_ch<<<grid_for((uint64_t)nVO * 32, 256, sms * 8), 256, 0, st>>>(
         d, VO.ptr, nVO, ch_up.ptr, ch_dn.ptr, ch_up_beg.ptr, ch_up_deg.ptr, ch_dn_beg.ptr,
-        ch_dn_deg.ptr, ch_up.count, ch_dn.count, true, r);
+        ch_dn_deg.ptr, ch_up.count, ch_dn.count, true, r, nullptr, 0, nullptr);
     CH_CHECK_LAUNCH();
     mark(&h->t_update_ms, e0);
     sync_ctl();
@@ -2865,7 +2996,10 @@ void Builder::run_rounds() {
     CH_CHECK_LAUNCH();
     hctl->nVO = n;
     CH_CUDA_TRY(cudaMemcpyAsync(&ctl.ptr->nVO, &hctl->nVO, 4, cudaMemcpyHostToDevice, st));
-    uint32_t nA = n, nVO = n;
+    CH_CUDA_TRY(cudaStreamSynchronize(st));  // k_contract_prep writes hctl from now on
+    k_round_begin<<<1, 1, 0, st>>>(ctl.ptr);
+    CH_CHECK_LAUNCH();
+    uint32_t nA = n, nVO = n, last_nS = n;
     uint64_t live_edges = h->m_input;
     // The statistics row of a round is finished at the next read of the
     // control block, which also brings the round's contraction counters
@@ -2890,17 +3024,18 @@ void Builder::run_rounds() {
     for (uint32_t r = 0; nVO > 0; ++r) {
         if (r > 0x7FFFFFF0u) throw Error{CH_ERANGE, "too many rounds"};
         cur_round = (int)r;
-        // reset per-round counters
-        k_round_begin<<<1, 1, 0, st>>>(ctl.ptr);
-        CH_CHECK_LAUNCH();
+        if (r && r % TS_ROUNDS == 0) fetch_stamps(r);
+        unsigned long long *ts = stamps.ptr + (size_t)(r % TS_ROUNDS) * TS_COUNT;
         // 1-2: score the affected set
-        cudaEvent_t e0 = start();
         const uint32_t sstamp = 2 * r + 1, cstamp = 2 * r + 2;
         if (nA) {
-            k_score_prep<<<grid_for((uint64_t)nA * 32, 256, sms * 8), 256, 0, st>>>(d, A.ptr, nA, sstamp,
-                                                                                    S.ptr, r);
-            CH_CHECK_LAUNCH();
-            witness<MODE_SCORE>(S.ptr, &ctl.ptr->nS, nA * 4 + 32 > n ? n : nA * 4 + 32, r);
+            launch_pdl(k_score_prep, grid_for((uint64_t)nA * 32, 256, sms * 8), 256, 0, st, d, A.ptr, nA, sstamp,
+                       S.ptr, r, ts + TS_SCORE);
+            witness<MODE_SCORE>(S.ptr, &ctl.ptr->nS, nA * 4 + 32 > n ? n : nA * 4 + 32, last_nS, r, ts + TS_WIT);
+            if (prune || tracing || learned || composite) {
+                k_stamp<<<1, 1, 0, st>>>(ts + TS_WIT_END);
+                CH_CHECK_LAUNCH();
+            }
             if (prune) {
                 // Alg. 3's pruning, then the scores on the pruned overlay from
                 // the recorded distances
@@ -2942,25 +3077,22 @@ void Builder::run_rounds() {
                 if (tracing) trace_count += nA;
             }
         }
-        mark(&h->t_score_ms, e0, 0);
-        // 3: select
-        e0 = start();
-        // about 16 warps an SM before a warp takes a second vertex
+        // 3: select, about 16 warps an SM before a warp takes a second vertex
         const uint32_t per = (uint32_t)std::min<uint64_t>(32, 1 + nVO / (16 * (uint64_t)sms));
-        k_select<<<grid_for((uint64_t)(nVO + per - 1) / per * 32, 256, sms * 8), 256, 0, st>>>(d, VO.ptr, nVO, per,
-                                                                                              r, F.ptr);
-        CH_CHECK_LAUNCH();
-        mark(&h->t_select_ms, e0, 1);
+        launch_pdl(k_select, grid_for((uint64_t)(nVO + per - 1) / per * 32, 256, sms * 8), 256, 0, st, d, VO.ptr, nVO,
+                   per, r, F.ptr, ts + TS_SELECT);
         // 4: contraction bookkeeping
-        e0 = start();
-        k_contract_prep<<<grid_for((uint64_t)nVO * 32, 256, sms * 8), 256, 0, st>>>(
-            d, F.ptr, cstamp, r + 1, S2.ptr, Anext.ptr);
-        CH_CHECK_LAUNCH();
-        mark(&h->t_prep_ms, e0, 2);
-        sync_ctl();
+        ++reads;
+        launch_pdl(k_contract_prep, grid_for((uint64_t)nVO * 32, 256, sms * 4), 256, 0, st, d, F.ptr, cstamp, r + 1,
+                   S2.ptr, Anext.ptr, ts + TS_PREP, box, reads);
+        wait_ctl();
         finish_row();  // the round before
         const Ctl c = *hctl;
         const uint32_t nF = c.nF, nS2 = c.nS2, nAnext = c.nAnext;
+        last_nS = c.nS;
+        // overflow of the score phase's middle tier decides the next two phases'
+        // launches: a few sources are left to the dense tier
+        use_big = (use_big ? c.nOvf1 : c.nOvf2) > 4;
         if (nF == 0) {
             // no eligible vertex left (only possible with a finite bound):
             // the live vertices are the core
@@ -3002,44 +3134,17 @@ void Builder::run_rounds() {
             d.out_arena = out_adj.count;
             d.in_arena = in_adj.count;
         }
-        k_contract_begin<<<1, 1, 0, st>>>(ctl.ptr);
-        CH_CHECK_LAUNCH();
         // 5: witness searches for V_F's candidates
-        e0 = start();
-        if (nS2) witness<MODE_PRUNE>(S2.ptr, &ctl.ptr->nS2, nS2, r);
-        mark(&h->t_contract_ms, e0, 3);
+        if (nS2) witness<MODE_PRUNE>(S2.ptr, &ctl.ptr->nS2, nS2, nS2, r, ts + TS_CONTRACT);
         // 6-10
-        e0 = start();
-        k_emit_ch<<<grid_for((uint64_t)nF * 32, 256, sms * 8), 256, 0, st>>>(
-            d, F.ptr, nF, ch_up.ptr, ch_dn.ptr, ch_up_beg.ptr, ch_up_deg.ptr, ch_dn_beg.ptr,
-            ch_dn_deg.ptr, ch_up.count, ch_dn.count, false, r);
-        CH_CHECK_LAUNCH();
-        if (nAnext) {
-            const int ga = grid_for(nAnext, 256, sms * 8);
-            const int gw = grid_for((uint64_t)nAnext * 32, 256, sms * 8);
-            k_compact_lists<<<gw, 256, 0, st>>>(d, Anext.ptr, nAnext, r);
-            CH_CHECK_LAUNCH();
-            k_reserve<<<ga, 256, 0, st>>>(d, Anext.ptr, nAnext, reqO.ptr, reqI.ptr);
-            CH_CHECK_LAUNCH();
-            exclusive_scan<uint64_t>(reqO.ptr, posO.ptr, nullptr, nAnext, reinterpret_cast<uint64_t *>(&ctl.ptr->relocOut),
-                                     scan64.ptr, st);
-            exclusive_scan<uint64_t>(reqI.ptr, posI.ptr, nullptr, nAnext, reinterpret_cast<uint64_t *>(&ctl.ptr->relocIn),
-                                     scan64.ptr, st);
-            k_relocate<<<gw, 256, 0, st>>>(d, Anext.ptr, nAnext, reqO.ptr, posO.ptr, reqI.ptr,
-                                           posI.ptr);
-            CH_CHECK_LAUNCH();
-        }
-        const uint64_t rec_bound = std::max<uint64_t>(cb, 1);
-        k_insert<<<grid_for(rec_bound, 256, sms * 8), 256, 0, st>>>(
-            d, rec.ptr, rec_flag.ptr, r, log.ptr, log_round.ptr);
-        CH_CHECK_LAUNCH();
-        compact_alive(VO.ptr, &ctl.ptr->nVO, nVO, level.ptr, VO2.ptr, &ctl.ptr->nVO2, tmp.ptr,
-                      scan32.ptr, st);
+        launch_pdl(k_emit_ch, grid_for(((uint64_t)nF + nAnext) * 32, 256, sms * 8), 256, 0, st, d, F.ptr, nF,
+                   ch_up.ptr, ch_dn.ptr, ch_up_beg.ptr, ch_up_deg.ptr, ch_dn_beg.ptr, ch_dn_deg.ptr, ch_up.count,
+                   ch_dn.count, false, r, Anext.ptr, nAnext, ts + TS_UPDATE);
+        launch_pdl(k_insert, grid_for(std::max<uint64_t>(cb, nVO), 256, sms * 8), 256, 0, st, d, rec.ptr,
+                   rec_flag.ptr, r, log.ptr, log_round.ptr, VO.ptr, nVO, VO2.ptr);
         std::swap(VO, VO2);
-        k_round_end<<<1, 1, 0, st>>>(ctl.ptr, nAnext ? 1 : 0);
-        CH_CHECK_LAUNCH();
+        launch_pdl(k_round_end, 1, 1, 0, st, ctl.ptr, ts + TS_END);
         std::swap(A, Anext);
-        mark(&h->t_update_ms, e0, 4);
         // this round's row: what is known now; its contraction counters
         // arrive with the next read of the control block
         row = {};
@@ -3072,6 +3177,7 @@ void Builder::run_rounds() {
         sync_ctl();
         finish_row();
     }
+    fetch_stamps((uint32_t)cur_round + 1);
     h->n_shortcuts = log_count;
     h->witness_bytes = 0;
 }
@@ -3156,6 +3262,25 @@ void Builder::postprocess() {
     CH_CUDA_TRY(cudaStreamSynchronize(st));  // before `rows` goes
 }
 
+// Shared-memory sizes and resident blocks of the block tiers' kernels.
+template <int FEAT, class SM, int MODE>
+int resolve_block_tier(int sms, int threads) {
+    const auto kern = k_witness_block<MODE, FEAT, SM>;
+    CH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM)));
+    int per_sm = 0;
+    CH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sizeof(SM)));
+    return sms * std::max(1, per_sm);
+}
+
+template <int FEAT>
+void resolve_block_tiers(Builder &b) {
+    resolve_block_tier<FEAT, BigSmem<MODE_SCORE>, MODE_SCORE>(b.sms, WB_THREADS);
+    b.big_blocks = resolve_block_tier<FEAT, BigSmem<MODE_PRUNE>, MODE_PRUNE>(b.sms, WB_THREADS);
+    resolve_block_tier<FEAT, MidSmem<MODE_PRUNE>, MODE_PRUNE>(b.sms, WM_THREADS_MANY);
+    b.mid_blocks = resolve_block_tier<FEAT, MidSmem<MODE_SCORE>, MODE_SCORE>(b.sms, WM_THREADS_MANY);
+    b.mid_blocks_few = b.sms * 2;
+}
+
 }  // namespace
 
 void build_hierarchy(ch_s *h, const ch_graph_t *g, const ch_params_t *p) {
@@ -3169,14 +3294,15 @@ void build_hierarchy(ch_s *h, const ch_graph_t *g, const ch_params_t *p) {
     const uint32_t n = g->n;
     h->n = n;
     h->hop_limit = p->hop_limit;
-    CH_CUDA_TRY(cudaMallocHost(&b.hctl, sizeof(Ctl)));
+    CH_CUDA_TRY(cudaMallocHost(&b.box, sizeof(HostBox)));
     struct PinnedFree {
-        Ctl *p;
+        HostBox *p;
         ~PinnedFree() {
             if (p) cudaFreeHost(p);
         }
-    } pf{b.hctl};
-    std::memset(b.hctl, 0, sizeof(Ctl));
+    } pf{b.box};
+    std::memset((void *)b.box, 0, sizeof(HostBox));
+    b.hctl = &b.box->c;
     b.ctl.alloc(1);
     b.ctl.zero(b.st);
     b.scan32.alloc(kScanScratch);
@@ -3219,45 +3345,22 @@ void build_hierarchy(ch_s *h, const ch_graph_t *g, const ch_params_t *p) {
     b.new_out.zero(b.st);
     b.new_in.alloc(n);
     b.new_in.zero(b.st);
-    for (auto *l : {&b.VO, &b.VO2, &b.A, &b.Anext, &b.S, &b.S2, &b.F, &b.ovf, &b.ovf2}) l->alloc(n);
+    for (auto *l : {&b.VO, &b.VO2, &b.A, &b.Anext, &b.S, &b.S2, &b.F, &b.ovf, &b.ovf1, &b.ovf2}) l->alloc(n);
     {
-        const int smem = (int)sizeof(BlkSmem);
-        CH_CUDA_TRY(cudaFuncSetAttribute(k_witness_block<MODE_SCORE, 0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        CH_CUDA_TRY(cudaFuncSetAttribute(k_witness_block<MODE_PRUNE, 0>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         const int feat = (p->witness_memo_limit || p->witness_prune ? F_XM : 0) |
                          (p->witness_level_work && !p->witness_settle_cap ? F_LW : 0) |
                          (p->witness_prune ? F_PR : 0) | (p->witness_settle_cap ? F_TH : 0);
-        auto set_smem = [&](auto score_kernel, auto prune_kernel) {
-            CH_CUDA_TRY(cudaFuncSetAttribute(score_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            CH_CUDA_TRY(cudaFuncSetAttribute(prune_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        };
-        if (feat == F_XM) set_smem(k_witness_block<MODE_SCORE, F_XM>, k_witness_block<MODE_PRUNE, F_XM>);
-        if (feat == F_LW) set_smem(k_witness_block<MODE_SCORE, F_LW>, k_witness_block<MODE_PRUNE, F_LW>);
-        if (feat == (F_XM | F_LW))
-            set_smem(k_witness_block<MODE_SCORE, F_XM | F_LW>, k_witness_block<MODE_PRUNE, F_XM | F_LW>);
-        if (feat == (F_XM | F_PR))
-            set_smem(k_witness_block<MODE_SCORE, F_XM | F_PR>, k_witness_block<MODE_PRUNE, F_XM | F_PR>);
-        if (feat == (F_XM | F_LW | F_PR))
-            set_smem(k_witness_block<MODE_SCORE, F_XM | F_LW | F_PR>,
-                     k_witness_block<MODE_PRUNE, F_XM | F_LW | F_PR>);
-        if (feat == F_TH) set_smem(k_witness_block<MODE_SCORE, F_TH>, k_witness_block<MODE_PRUNE, F_TH>);
-        if (feat == (F_TH | F_XM))
-            set_smem(k_witness_block<MODE_SCORE, F_TH | F_XM>, k_witness_block<MODE_PRUNE, F_TH | F_XM>);
-        if (feat == (F_TH | F_XM | F_PR))
-            set_smem(k_witness_block<MODE_SCORE, F_TH | F_XM | F_PR>,
-                     k_witness_block<MODE_PRUNE, F_TH | F_XM | F_PR>);
-        int per_sm = 0;
-        CH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_witness_block<MODE_PRUNE, 0>,
-                                                                  WB_THREADS, smem));
-        b.blk_blocks = b.sms * std::max(1, per_sm);
+        switch (feat) {
+            case F_XM: resolve_block_tiers<F_XM>(b); break;
+            case F_LW: resolve_block_tiers<F_LW>(b); break;
+            case F_XM | F_LW: resolve_block_tiers<F_XM | F_LW>(b); break;
+            case F_XM | F_PR: resolve_block_tiers<F_XM | F_PR>(b); break;
+            case F_XM | F_LW | F_PR: resolve_block_tiers<F_XM | F_LW | F_PR>(b); break;
+            default: resolve_block_tiers<0>(b); break;
+        }
     }
-    b.tmp.alloc((size_t)n + 1);
-    b.reqO.alloc(n);
-    b.reqI.alloc(n);
-    b.posO.alloc(n);
-    b.posI.alloc(n);
+    b.stamps.alloc((size_t)TS_ROUNDS * TS_COUNT);
+    b.stamps.zero(b.st);
     const uint64_t m1 = h->m_input;
     b.rec.alloc(std::max<uint64_t>(1024, m1));
     b.rec_flag.alloc(b.rec.count);
@@ -3387,13 +3490,26 @@ void build_hierarchy(ch_s *h, const ch_graph_t *g, const ch_params_t *p) {
     b.mark(&h->stats.build_ms, t0);
     CH_CUDA_TRY(cudaStreamSynchronize(b.st));
 
-    h->round_times.assign(h->round_stats.size(), {});
     for (const Span &s : b.spans) {
         float ms = 0;
         CH_CUDA_TRY(cudaEventElapsedTime(&ms, s.a, s.b));
         *s.acc += ms;
-        if (s.round >= 0 && s.phase >= 0 && (size_t)s.round < h->round_times.size())
-            h->round_times[s.round][s.phase] += ms;
+    }
+    // times of the rounds' steps from their stamps (a step that did not run,
+    // or whose end did not, has none)
+    h->round_times.assign(h->round_stats.size(), {});
+    for (size_t r = 0; r < b.hstamps.size() / TS_COUNT; ++r) {
+        const unsigned long long *t = b.hstamps.data() + r * TS_COUNT;
+        auto ms = [&](int from, int to) { return t[from] && t[to] > t[from] ? (double)(t[to] - t[from]) * 1e-6 : 0.0; };
+        const double wit = ms(TS_WIT, t[TS_WIT_END] ? TS_WIT_END : TS_SELECT), contract = ms(TS_CONTRACT, TS_UPDATE);
+        const double row[CH_NTIME] = {ms(TS_SCORE, TS_SELECT), ms(TS_SELECT, TS_PREP), ms(TS_PREP, TS_PREP_END),
+                                      contract,                ms(TS_UPDATE, TS_END),  wit + contract};
+        double *acc[CH_NTIME] = {&h->t_score_ms,    &h->t_select_ms, &h->t_prep_ms,
+                                 &h->t_contract_ms, &h->t_update_ms, &h->t_witness_ms};
+        for (uint32_t k = 0; k < CH_NTIME; ++k) {
+            *acc[k] += row[k];
+            if (r < h->round_times.size()) h->round_times[r][k] = row[k];
+        }
     }
     const Ctl &c = *b.hctl;
     h->stats.witness_sources = c.wit_sources + c.wit_block + c.wit_fallback;
