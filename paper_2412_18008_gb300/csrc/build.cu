@@ -1115,6 +1115,13 @@ using MidSmem = BlkSmem<10, 512, 9, MODE>;
 template <int MODE>
 using BigSmem = BlkSmem<12, 2048, 11, MODE>;
 
+// Entries a warp takes at a time when a block's warps share `count` of them:
+// all warps get some (a frontier of 100 vertices would keep 4 of 16 warps busy
+// at 32 a warp), at most 32 each.
+__device__ __forceinline__ uint32_t block_share(uint32_t count, uint32_t nwarps) {
+    return min(32u, max(1u, (count + nwarps - 1) / nwarps));
+}
+
 // The sources of a block tier's launch, and where it hands on those it cannot
 // hold (hubs go to the dense tier's list at once).
 struct BlkList {
@@ -1176,12 +1183,13 @@ __global__ void __launch_bounds__(SM::THREADS, SM::TB < 12 ? 2 : 1) k_witness_bl
         __syncthreads();
         // Phase 0: heaviest candidate weight of the source, and whether every
         // contracted middle has its score-phase decisions memoised. Each warp
-        // takes 32 of the source's out-edges and spreads their middles'
+        // takes its share of the source's out-edges and spreads their middles'
         // out-lists over its lanes.
+        const uint32_t share = block_share(sd, nwarps);
         uint32_t lb = 0;
-        for (uint32_t c0 = warp * 32; c0 < sd; c0 += nwarps * 32) {
+        for (uint32_t c0 = warp * share; c0 < sd; c0 += nwarps * share) {
             const uint32_t j = c0 + lane;
-            const bool valid = j < sd;
+            const bool valid = lane < share && j < sd;
             const uint2 e = valid ? d.out_adj[sb + j] : make_uint2(0, 0);
             const bool mid = valid && id_ok(d, e.x) && is_middle<MODE>(d, e.x, r);
             if (MODE == MODE_PRUNE && mid && d.kround[e.x] != r + 1) b.memo_ok = 0;
@@ -1278,9 +1286,10 @@ __global__ void __launch_bounds__(SM::THREADS, SM::TB < 12 ? 2 : 1) k_witness_bl
                 if constexpr (LW) b.lwork = 0;
             }
             __syncthreads();
-            for (uint32_t f0 = warp * 32; f0 < nfront; f0 += nwarps * 32) {
+            const uint32_t fshare = block_share(nfront, nwarps);
+            for (uint32_t f0 = warp * fshare; f0 < nfront; f0 += nwarps * fshare) {
                 const uint32_t fi = f0 + lane;
-                const bool fv = fi < nfront && fi < (uint32_t)SM::FC;
+                const bool fv = lane < fshare && fi < nfront && fi < (uint32_t)SM::FC;
                 const uint2 fe = fv ? b.front[cur][fi] : make_uint2(0, 0);
                 const bool fok = fv && fe.x < (uint32_t)SM::T;
                 if (fv && !fok) atomicOr(&ctl->err, ERR_BOUND);
@@ -1337,10 +1346,10 @@ __global__ void __launch_bounds__(SM::THREADS, SM::TB < 12 ? 2 : 1) k_witness_bl
             if (tid == 0) l.out[atomicAdd(l.out_cnt, 1u)] = s;
             continue;
         }
-        // Phase 2: decisions, each warp taking 32 of the source's out-edges.
-        for (uint32_t c0 = warp * 32; c0 < sd; c0 += nwarps * 32) {
+        // Phase 2: decisions, each warp taking its share of the source's out-edges.
+        for (uint32_t c0 = warp * share; c0 < sd; c0 += nwarps * share) {
             const uint32_t j = c0 + lane;
-            const bool valid = j < sd;
+            const bool valid = lane < share && j < sd;
             const uint2 e = valid ? d.out_adj[sb + j] : make_uint2(0, 0);
             const bool mid = valid && id_ok(d, e.x) && is_middle<MODE>(d, e.x, r);
             uint32_t cnt = mid ? d.out_deg[e.x] : 0;
@@ -1449,9 +1458,9 @@ __global__ void __launch_bounds__(SM::THREADS, SM::TB < 12 ? 2 : 1) k_witness_bl
         if constexpr (XM) {
             if (bound != 0) {
                 bool full = false;
-                for (uint32_t c0 = warp * 32; c0 < sd; c0 += nwarps * 32) {
+                for (uint32_t c0 = warp * share; c0 < sd; c0 += nwarps * share) {
                     const uint32_t j = c0 + lane;
-                    const bool valid = j < sd;
+                    const bool valid = lane < share && j < sd;
                     const uint2 e = valid ? d.out_adj[sb + j] : make_uint2(0, 0);
                     const bool mid = valid && id_ok(d, e.x) && is_middle<MODE>(d, e.x, r);
                     uint32_t cnt = mid ? d.out_deg[e.x] : 0;
@@ -2109,23 +2118,30 @@ __global__ void k_contract_prep(Dev d, const uint32_t *F, uint32_t src_stamp, ui
 constexpr uint32_t TOMB = 0xFFFFFFFFu;  // a pruned adjacency entry (never a vertex id)
 
 // Stable in-place removal, by one warp, of this round's contracted vertices
-// and of pruned entries (tombstones) from a list (32 entries per step;
+// and of pruned entries (tombstones) from a list (128 entries per step;
 // writes never pass the reads).
 __device__ __forceinline__ uint32_t warp_compact_list(const Dev &d, uint2 *adj, uint64_t b, uint32_t dg,
                                                       uint32_t r) {
     const uint32_t lane = lane_id();
+    constexpr uint32_t U = 4;  // entries a lane has in flight (a hub's list is thousands of steps long)
     uint32_t k = 0;
-    for (uint32_t j0 = 0; j0 < dg; j0 += 32) {
-        const uint32_t j = j0 + lane;
-        uint2 e = make_uint2(0, 0);
-        bool keep = false;
-        if (j < dg) {
-            e = adj[b + j];
-            keep = e.x != TOMB && id_ok(d, e.x) && d.level[e.x] != r;
+    for (uint32_t j0 = 0; j0 < dg; j0 += 32 * U) {
+        uint2 e[U];
+        bool keep[U];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) {
+            const uint32_t j = j0 + 32 * u + lane;
+            e[u] = j < dg ? adj[b + j] : make_uint2(TOMB, 0);
         }
-        const uint32_t m = __ballot_sync(FULL, keep);
-        if (keep) adj[b + k + __popc(m & ((1u << lane) - 1u))] = e;
-        k += __popc(m);
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) keep[u] = e[u].x != TOMB && id_ok(d, e[u].x) && d.level[e[u].x] != r;
+        __syncwarp();  // the group is read before any of it is written
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) {
+            const uint32_t m = __ballot_sync(FULL, keep[u]);
+            if (keep[u]) adj[b + k + __popc(m & ((1u << lane) - 1u))] = e[u];
+            k += __popc(m);
+        }
         __syncwarp();
     }
     return k;
@@ -2163,7 +2179,19 @@ __device__ __forceinline__ void update_lists(const Dev &d, uint32_t x, uint32_t 
         if (lane == 0) nb = atomicAdd(tail, (unsigned long long)want);
         nb = __shfl_sync(FULL, nb, 0);
         if (!ok(nb, want)) continue;
-        for (uint32_t j = lane; j < k; j += 32) adj[nb + j] = adj[b + j];
+        for (uint32_t j0 = 0; j0 < k; j0 += 128) {
+            uint2 e[4];
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u) {
+                const uint32_t j = j0 + 32 * u + lane;
+                if (j < k) e[u] = adj[b + j];
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u) {
+                const uint32_t j = j0 + 32 * u + lane;
+                if (j < k) adj[nb + j] = e[u];
+            }
+        }
         __syncwarp();
         if (lane == 0) {
             beg[x] = nb;
@@ -2413,6 +2441,29 @@ __global__ void k_round_end(Ctl *ctl, unsigned long long *ts) {
     round_begin(ctl);
 }
 
+// Each lane's list [b, b + n): sets the weight of its first entry for v to w. A
+// thread walks a list of up to 128 entries, the warp together a longer one.
+__device__ __forceinline__ void warp_lower_entry(uint2 *adj, uint64_t b, uint32_t n, uint32_t v, uint32_t w) {
+    const uint32_t lane = lane_id();
+    if (n <= 128)
+        for (uint32_t j = 0; j < n; ++j)
+            if (adj[b + j].x == v) {
+                adj[b + j].y = w;
+                break;
+            }
+    for (uint32_t m = __ballot_sync(FULL, n > 128); m; m &= m - 1) {
+        const uint32_t o = __ffs(m) - 1;
+        const uint64_t ob = __shfl_sync(FULL, b, o);
+        const uint32_t on = __shfl_sync(FULL, n, o), ov = __shfl_sync(FULL, v, o), ow = __shfl_sync(FULL, w, o);
+        for (uint32_t j0 = 0; j0 < on; j0 += 32) {
+            const uint32_t hit = __ballot_sync(FULL, j0 + lane < on && adj[ob + j0 + lane].x == ov);
+            if (!hit) continue;
+            if (lane == (uint32_t)__ffs(hit) - 1) adj[ob + j0 + lane].y = ow;
+            break;
+        }
+    }
+}
+
 // The round's shortcuts into the lists and the log; and, in the same launch,
 // the live vertices (level still INF) of VO into VO2, in any order: the kernels
 // that read the list only form sets from it.
@@ -2429,28 +2480,25 @@ __global__ void k_insert(Dev d, const uint4 *rec, const uint8_t *flag, uint32_t 
     }
     const uint32_t nRec = d.ctl->nRec;
     const uint64_t log_base = d.ctl->log_tail;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nRec;
-         i += gridDim.x * blockDim.x) {
-        const uint4 c = rec[i];  // (v1, v2, w, via)
-        if (!id_ok(d, c.x) || !id_ok(d, c.y)) continue;
-        if (flag[i]) {
-            // Lower an existing edge. It sits among the list's entries from
-            // before this kernel, ahead of anything appended concurrently.
-            const uint64_t ob = d.out_beg[c.x];
-            const uint32_t oc = out_list_ok(d, ob, d.out_cap[c.x]) ? d.out_cap[c.x] : 0;
-            for (uint32_t j = 0; j < oc; ++j)
-                if (d.out_adj[ob + j].x == c.y) {
-                    d.out_adj[ob + j].y = c.z;
-                    break;
-                }
-            const uint64_t ib = d.in_beg[c.y];
-            const uint32_t ic = in_list_ok(d, ib, d.in_cap[c.y]) ? d.in_cap[c.y] : 0;
-            for (uint32_t j = 0; j < ic; ++j)
-                if (d.in_adj[ib + j].x == c.x) {
-                    d.in_adj[ib + j].y = c.z;
-                    break;
-                }
-        } else {
+    for (uint32_t i0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; i0 < nRec; i0 += nthreads) {
+        const uint32_t i = i0 + lane_id();
+        const uint4 c = i < nRec ? rec[i] : make_uint4(0, 0, 0, 0);  // (v1, v2, w, via)
+        const bool ok = i < nRec && id_ok(d, c.x) && id_ok(d, c.y);
+        const bool lower = ok && flag[i];
+        // Lower an existing edge. It sits among the list's entries from before
+        // this kernel, ahead of anything appended concurrently.
+        uint64_t ob = 0, ib = 0;
+        uint32_t oc = 0, ic = 0;
+        if (lower) {
+            ob = d.out_beg[c.x];
+            oc = out_list_ok(d, ob, d.out_cap[c.x]) ? d.out_cap[c.x] : 0;
+            ib = d.in_beg[c.y];
+            ic = in_list_ok(d, ib, d.in_cap[c.y]) ? d.in_cap[c.y] : 0;
+        }
+        warp_lower_entry(d.out_adj, ob, oc, c.y, c.z);
+        warp_lower_entry(d.in_adj, ib, ic, c.x, c.z);
+        if (!ok) continue;
+        if (!lower) {
             const uint32_t p = atomicAdd(&d.out_deg[c.x], 1u);
             if (p < d.out_cap[c.x] && out_list_ok(d, d.out_beg[c.x], p + 1))
                 d.out_adj[d.out_beg[c.x] + p] = make_uint2(c.y, c.z);
@@ -2466,10 +2514,6 @@ __global__ void k_insert(Dev d, const uint4 *rec, const uint8_t *flag, uint32_t 
         log_round[log_base + i] = r;
     }
 }
-
-// --------------------------------------------------------------------------
-// Postprocess: rank by (level, score, id) and the rank-ordered CSRs
-// --------------------------------------------------------------------------
 
 __global__ void k_rank_keys(const uint32_t *level, const int32_t *P, uint32_t n, uint64_t *keys,
                             uint32_t *vals) {
@@ -2495,21 +2539,34 @@ constexpr uint32_t RANKED_SORT_MAX = 64;  // longest row a thread insertion-sort
 constexpr uint32_t ROW_SORT_MAX = 16384;  // longest row a block sorts in shared memory (8 B an entry)
 constexpr int ROW_SORT_THREADS = 512;
 
-// Sorts the listed rows of a rank-ordered CSR by target rank, a block a row: a
-// bitonic sort in shared memory of target << 32 | weight (targets of a row are
-// distinct), padded to a power of two with ones. Rows above ROW_SORT_MAX are
-// left. An RMAT 2^17 hierarchy (5.3M entries in both CSRs, rows of up to 10^4):
-// well under 1 ms, against 6.3 for a radix sort of both whole CSRs.
+// Fills and sorts the listed rows of a rank-ordered CSR, a block a row: the
+// vertex's edges with their targets' ranks go to shared memory, are sorted there
+// as target << 32 | weight (bitonic; targets of a row are distinct; padded to a
+// power of two with ones) and written. Rows above ROW_SORT_MAX are filled
+// unsorted. An RMAT 2^17 hierarchy (5.3M entries in both CSRs, rows of up to
+// 10^4): 0.9 ms, against 6.1 for a thread filling each row and 6.3 for a radix
+// sort of both whole CSRs.
 __global__ void __launch_bounds__(ROW_SORT_THREADS)
-k_sort_rows(const uint32_t *rows, const uint32_t *off, uint2 *adj) {
+k_sort_rows(const uint32_t *rows, const uint32_t *perm, const uint32_t *rank, uint32_t n, const uint64_t *beg,
+            const uint2 *src, const uint32_t *off, uint2 *adj, Ctl *ctl) {
     extern __shared__ unsigned long long row_smem[];
     const uint32_t i = rows[blockIdx.x];
     const uint32_t b = off[i], m = off[i + 1] - b;
-    if (m > ROW_SORT_MAX) return;
+    const uint2 *from = src + beg[perm[i]];  // in range: k_ranked_fill listed the row
+    auto entry = [&](uint32_t j) {
+        const uint2 e = from[j];
+        if (e.x < n) return make_uint2(rank[e.x], e.y);
+        atomicOr(&ctl->err, ERR_BOUND);
+        return make_uint2(0, INF);
+    };
+    if (m > ROW_SORT_MAX) {
+        for (uint32_t j = threadIdx.x; j < m; j += ROW_SORT_THREADS) adj[b + j] = entry(j);
+        return;
+    }
     uint32_t n2 = 2;
     while (n2 < m) n2 <<= 1;
     for (uint32_t j = threadIdx.x; j < n2; j += ROW_SORT_THREADS) {
-        const uint2 a = j < m ? adj[b + j] : make_uint2(INF, INF);
+        const uint2 a = j < m ? entry(j) : make_uint2(INF, INF);
         row_smem[j] = ((unsigned long long)a.x << 32) | a.y;
     }
     for (uint32_t size = 2; size <= n2; size <<= 1)
@@ -2567,6 +2624,14 @@ __global__ void k_ranked_fill(const uint32_t *perm, const uint32_t *rank, uint32
             atomicOr(&ctl->err, ERR_BOUND);
             continue;
         }
+        // rows are sorted by target rank, which makes the list order
+        // canonical: short rows here (insertion sort), longer ones are listed
+        // for k_sort_rows
+        if (dg > RANKED_SORT_MAX) {
+            rows[atomicAdd(&ctl->longRows[dir], 1u)] = i;
+            atomicMax(&ctl->longest[dir], dg);
+            continue;
+        }
         uint2 *out = dst + off[i];
         for (uint32_t j = 0; j < dg; ++j) {
             const uint2 e = src[b + j];
@@ -2576,14 +2641,6 @@ __global__ void k_ranked_fill(const uint32_t *perm, const uint32_t *rank, uint32
                 continue;
             }
             out[j] = make_uint2(rank[e.x], e.y);
-        }
-        // rows are sorted by target rank, which makes the list order
-        // canonical: short rows here (insertion sort), longer ones are listed
-        // for k_sort_rows or, above what a block sorts, for the radix sort
-        if (dg > RANKED_SORT_MAX) {
-            rows[atomicAdd(&ctl->longRows[dir], 1u)] = i;
-            atomicMax(&ctl->longest[dir], dg);
-            continue;
         }
         for (uint32_t j = 1; j < dg; ++j) {
             const uint2 t = out[j];
@@ -2610,6 +2667,9 @@ int bits_for(uint64_t x) {
 // Phases of up to this many sources an SM skip the warp tier (1M-vertex
 // geometric build: 60 ms with 64, 66 with 16; with 160, 2% slower than 64).
 constexpr uint32_t DIRECT_SOURCES = 64;
+// And with up to this many, a source gets 512 threads instead of 128 (1M-vertex
+// build: 47.4 ms with 6, 49.2 with 2; 256 threads: 48.8).
+constexpr uint32_t FEW_SOURCES = 6;
 
 struct EventPool {
     std::vector<cudaEvent_t> evs;
@@ -2922,7 +2982,7 @@ void Builder::launch_witness(const WArgs &a, uint32_t nS_max, uint32_t expected)
         ++h->witness_launches;
     }
     if constexpr (!TH) {
-        const bool few = direct && expected <= 2 * (uint32_t)sms;
+        const bool few = direct && expected <= FEW_SOURCES * (uint32_t)sms;
         BlkList mid{direct ? a.S : ovf.ptr, direct ? a.nS : &c->nOvf, &c->work3, ovf1.ptr, &c->nOvf1,
                     direct ? a.ts : nullptr};
         const BlkList big{ovf1.ptr, &c->nOvf1, &c->work4, ovf2.ptr, &c->nOvf2, nullptr};
@@ -3231,15 +3291,15 @@ void Builder::postprocess() {
         DevBuf<uint2> &adj = dir == 0 ? h->up_adj : h->dn_adj;
         const uint64_t m = dir == 0 ? n_up : n_dn;
         if (!hctl->longRows[dir]) continue;
-        if (hctl->longest[dir] <= ROW_SORT_MAX) {
-            uint32_t n2 = 2;
-            while (n2 < hctl->longest[dir]) n2 <<= 1;
-            const int smem = (int)(n2 * sizeof(unsigned long long));
-            CH_CUDA_TRY(cudaFuncSetAttribute(k_sort_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            k_sort_rows<<<hctl->longRows[dir], ROW_SORT_THREADS, smem, st>>>(rows.ptr + (size_t)dir * n, off.ptr,
-                                                                             adj.ptr);
-            CH_CHECK_LAUNCH();
-        } else {
+        uint32_t n2 = 2;
+        while (n2 < std::min(hctl->longest[dir], ROW_SORT_MAX)) n2 <<= 1;
+        const int smem = (int)(n2 * sizeof(unsigned long long));
+        CH_CUDA_TRY(cudaFuncSetAttribute(k_sort_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        k_sort_rows<<<hctl->longRows[dir], ROW_SORT_THREADS, smem, st>>>(
+            rows.ptr + (size_t)dir * n, h->perm.ptr, h->rank.ptr, n, dir == 0 ? ch_up_beg.ptr : ch_dn_beg.ptr,
+            dir == 0 ? ch_up.ptr : ch_dn.ptr, off.ptr, adj.ptr, ctl.ptr);
+        CH_CHECK_LAUNCH();
+        if (hctl->longest[dir] > ROW_SORT_MAX) {
             // sort every row of the CSR at once by (row, target rank)
             std::vector<int> rd;
             append_digits(rd, 0, bits_for(n));
@@ -3259,7 +3319,7 @@ void Builder::postprocess() {
             CH_CUDA_TRY(cudaStreamSynchronize(st));
         }
     }
-    CH_CUDA_TRY(cudaStreamSynchronize(st));  // before `rows` goes
+    if (hctl->longRows[0] || hctl->longRows[1]) sync_ctl();  // (and before `rows` goes)
 }
 
 // Shared-memory sizes and resident blocks of the block tiers' kernels.
