@@ -281,10 +281,15 @@ __device__ uint32_t sv_query(const SvArgs &a, const Tab &t, uint32_t rs, uint32_
     return res;
 }
 
-template <bool WARP, bool STALL, bool DELTA = false>
-__global__ void __launch_bounds__(QB_THREADS) k_serve(SvArgs a) {
+// Positions a block takes at once while the backlog is long (at least twice that
+// many for every block): the counter and the published count are read once for
+// all of them, and the descriptor once for the targets of one request.
+constexpr uint32_t SV_TAKE = 4;
+
+template <bool WARP, bool STALL, bool DELTA = false, int TB = 12>
+__global__ void __launch_bounds__(QB_THREADS, TB == 11 ? 6 : 1) k_serve(SvArgs a) {
     extern __shared__ __align__(16) unsigned char qb_raw[];
-    QBSmem<12> &q = *reinterpret_cast<QBSmem<12> *>(qb_raw);
+    QBSmem<TB> &q = *reinterpret_cast<QBSmem<TB> *>(qb_raw);
     QStat stat;  // not reported
     qb_clear(q);
     __shared__ uint32_t s_go, s_src, s_tgt, s_k, s_slot, s_first;
@@ -302,6 +307,9 @@ __global__ void __launch_bounds__(QB_THREADS) k_serve(SvArgs a) {
     t.front = a.front + blockIdx.x * (size_t)a.fcap * 2;
     t.mask = (uint32_t)tsz - 1;
     t.fcap = a.fcap;
+    unsigned long long next = 0, end = 0;  // thread 0: positions taken and not yet served
+    uint32_t seen = 0;                     // thread 0: entry (ticket + 1) whose descriptor s_* hold
+    uint64_t seen_pos = 0;
     while (true) {
         __syncthreads();
         // Thread 0 takes the next published pool position. A position is
@@ -315,13 +323,20 @@ __global__ void __launch_bounds__(QB_THREADS) k_serve(SvArgs a) {
             const unsigned long long t0 = globaltimer();
             unsigned sleep_ns = 256;
             unsigned long long pos = 0;
-            while (true) {
+            if (next < end) {
+                pos = next++;
+                s_go = 1;
+            }
+            while (!s_go) {
                 if (*(volatile uint32_t *)a.closing == a.epoch) break;
                 const unsigned long long pub = ld_acquire_sys(&a.ctl->published);
                 const unsigned long long c = *(volatile unsigned long long *)a.claimed;
                 if (c < pub) {
-                    if (atomicCAS(a.claimed, c, c + 1ull) == c) {
+                    const uint32_t take = pub - c >= 2ull * SV_TAKE * gridDim.x ? SV_TAKE : 1u;
+                    if (atomicCAS(a.claimed, c, c + take) == c) {
                         pos = c;
+                        next = c + 1;
+                        end = c + take;
                         s_go = 1;
                         break;
                     }
@@ -359,6 +374,13 @@ __global__ void __launch_bounds__(QB_THREADS) k_serve(SvArgs a) {
                 uint64_t dseq = 0, dpos = 0;
                 while (true) {
                     v = ld_sys(a.item_req + e);
+                    if (v != 0 && v == seen && pos < seen_pos + s_k) {
+                        // another target of the request served last
+                        s_first = 0;
+                        s_tgt = ld_sys(a.targets + e);
+                        s_e = e;
+                        break;
+                    }
                     if (v != 0) {
                         const uint32_t slot = (v - 1) % a.ring;
                         const SvDesc *d = a.desc + slot;
@@ -374,6 +396,8 @@ __global__ void __launch_bounds__(QB_THREADS) k_serve(SvArgs a) {
                             s_slot = slot;
                             s_e = e;
                             if (s_first) a.t_begin[slot] = globaltimer();
+                            seen = v;
+                            seen_pos = dpos;
                             break;
                         }
                     }
@@ -403,7 +427,7 @@ __global__ void __launch_bounds__(QB_THREADS) k_serve(SvArgs a) {
             const uint32_t rs = g.rank[s], rt = g.rank[tv];
             if (rs < g.n && rt < g.n) {
                 uint32_t cnt;
-                if (!block_query<true, WARP, 12, STALL, DELTA>(q, g, rs, rt, ans, cnt, stat))
+                if (!block_query<true, WARP, TB, STALL, DELTA>(q, g, rs, rt, ans, cnt, stat))
                     ans = sv_query(a, t, rs, rt, q.cnt3, &q.ovf, &q.mu, &q.cnt);
             } else if (tid == 0) {
                 atomicOr(a.status, QERR_BOUND);
@@ -479,15 +503,18 @@ struct ch_server_s {
     gbch::SvArgs args{};
     void (*kern)(gbch::SvArgs) = nullptr;
     int threads = 0;
+    size_t smem = 0;
     uint32_t launches = 0;
 };
 
 namespace gbch {
 
+constexpr uint32_t SV_SMALL_N = 400000;
+
 // Launches the device loop for the next epoch.
 void server_launch(ch_server_s *sv) {
     sv->args.epoch = ++sv->launches;
-    sv->kern<<<sv->nblocks, sv->threads, sizeof(QBSmem<12>), sv->st>>>(sv->args);
+    sv->kern<<<sv->nblocks, sv->threads, sv->smem, sv->st>>>(sv->args);
     CH_CHECK_LAUNCH();
 }
 
@@ -500,12 +527,20 @@ void server_start(ch_server_s *sv, ch_s *h, const ch_server_params_t *p) {
     // the handle's query configuration (layout and block size)
     const bool warp = h->q_layout == CH_QUERY_WARP_FLAT;
     const int threads = (int)h->q_threads;
-    auto kern = warp ? (h->q_stall ? (h->q_delta ? k_serve<true, true, true> : k_serve<true, true>)
+    // The searches of hierarchies of up to SV_SMALL_N vertices fit 2^11-slot
+    // tables, which put six blocks on an SM instead of three (256K vertices, a
+    // burst of 80,000 pairs: 26.9 -> 11.1 ms, SV_TAKE included). Larger ones
+    // keep 2^12: a pair that overflows is redone on the block's slower global
+    // table.
+    const bool small = warp && h->q_stall && h->q_delta && h->n <= SV_SMALL_N;
+    auto kern = warp ? (h->q_stall ? (h->q_delta ? (small ? k_serve<true, true, true, 11> : k_serve<true, true, true>)
+                                                 : k_serve<true, true>)
                                    : k_serve<true, false>)
                      : k_serve<false, false>;
-    CH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(QBSmem<12>)));
+    sv->smem = small ? sizeof(QBSmem<11>) : sizeof(QBSmem<12>);
+    CH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv->smem));
     int per_sm = 0;
-    CH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sizeof(QBSmem<12>)));
+    CH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sv->smem));
     sv->nblocks = p->blocks ? p->blocks : (uint32_t)sms * (uint32_t)std::max(per_sm, 1);
     uint32_t tbits = 10;
     while (tbits < 24 && ((1u << tbits) < std::min<uint32_t>(h->n, 1u << 17))) ++tbits;
