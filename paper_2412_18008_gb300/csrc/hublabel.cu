@@ -25,14 +25,16 @@
 namespace gbch {
 namespace {
 
-// Batches of at least 2^14 and 60 sqrt(n) queries use labels. Labels cost a
+// Batches of at least 2^14 and 80 sqrt(n) queries use labels. Labels cost a
 // chain of launches and the labels of the upper levels whatever the batch, a
 // search costs the same for every query; measured (ms, labels / searches):
 // n = 20K: 17K queries 0.71 / 0.81; 100K: 20K queries 1.38 / 1.42, 30K 1.43 /
 // 2.04; 256K: 20K queries 2.7 / 2.2, 30K 2.8 / 3.1; 1M: 48K queries 9.0 / 9.0,
-// 64K 9.3 / 12.0, 1M queries 17.0 / 186.6.
+// 64K 9.3 / 12.0, 1M queries 17.0 / 186.6. (On hierarchies with quicker searches,
+// composite or memoised, the ways cross later: 100K memoised, 17K queries 1.38 /
+// 1.25; the line lies where labels win on all of them.)
 constexpr uint64_t HL_MIN_K = 1u << 14;
-constexpr uint64_t HL_MIN_SQRT = 60;
+constexpr uint64_t HL_MIN_SQRT = 80;
 bool batch_is_large(uint64_t k, uint32_t n) {
     return k >= HL_MIN_K && (k >= (1ull << 32) || k * k >= HL_MIN_SQRT * HL_MIN_SQRT * n);
 }

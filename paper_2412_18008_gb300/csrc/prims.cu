@@ -1,4 +1,4 @@
-// Device-wide scan, compaction and radix sort used by the build.
+// Device-wide scan and radix sort used by the build.
 #include "prims.cuh"
 
 namespace gbch {
@@ -96,25 +96,6 @@ __global__ void scan_apply_kernel(const T *in, T *out, const uint32_t *d_count,
     }
 }
 
-__global__ void alive_flags_kernel(const uint32_t *in, const uint32_t *d_count,
-                                   const uint32_t *level, uint32_t *flags) {
-    uint32_t count = *d_count;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += gridDim.x * blockDim.x)
-        flags[i] = level[in[i]] == INF ? 1u : 0u;
-}
-
-__global__ void alive_scatter_kernel(const uint32_t *in, const uint32_t *d_count,
-                                     const uint32_t *level, const uint32_t *pos,
-                                     uint32_t *out) {
-    uint32_t count = *d_count;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += gridDim.x * blockDim.x) {
-        uint32_t v = in[i];
-        if (level[v] == INF) out[pos[i]] = v;
-    }
-}
-
 constexpr int RS_THREADS = 256;
 
 __global__ void radix_hist_kernel(const uint64_t *keys, uint64_t n, int shift,
@@ -197,17 +178,6 @@ template void exclusive_scan<uint32_t>(const uint32_t *, uint32_t *, const uint3
                                        uint32_t *, uint32_t *, cudaStream_t);
 template void exclusive_scan<uint64_t>(const uint64_t *, uint64_t *, const uint32_t *, uint64_t,
                                        uint64_t *, uint64_t *, cudaStream_t);
-
-void compact_alive(const uint32_t *in, const uint32_t *d_in_count, uint64_t max_count,
-                   const uint32_t *level, uint32_t *out, uint32_t *d_out_count,
-                   uint32_t *tmp, uint32_t *scratch, cudaStream_t st) {
-    int g = grid_for(max_count, 256, 4 * 152 * 4);
-    alive_flags_kernel<<<g, 256, 0, st>>>(in, d_in_count, level, tmp);
-    CH_CHECK_LAUNCH();
-    exclusive_scan<uint32_t>(tmp, tmp, d_in_count, 0, d_out_count, scratch, st);
-    alive_scatter_kernel<<<g, 256, 0, st>>>(in, d_in_count, level, tmp, out);
-    CH_CHECK_LAUNCH();
-}
 
 void append_digits(std::vector<int> &digits, int lo_bit, int nbits) {
     if (nbits <= 0) return;

@@ -1,5 +1,5 @@
-// Device-wide primitives: exclusive scan, stable list compaction, LSD radix
-// sort of (uint64 key, uint32 value) pairs. All are stable and deterministic.
+// Device-wide primitives: exclusive scan, LSD radix sort of (uint64 key,
+// uint32 value) pairs. Both are stable and deterministic.
 #pragma once
 
 #include "common.cuh"
@@ -18,13 +18,6 @@ constexpr int kScanScratch = 1024;
 template <class T>
 void exclusive_scan(const T *in, T *out, const uint32_t *d_count, uint64_t host_count,
                     T *d_total, T *scratch, cudaStream_t st);
-
-// out[i] = in-list element kept in order where keep(level[v]) holds:
-// keeps ids v of `in` (count *d_in_count) with level[v] == INF; writes the
-// kept count to *d_out_count. `tmp` must hold max_count + 1 uint32.
-void compact_alive(const uint32_t *in, const uint32_t *d_in_count, uint64_t max_count,
-                   const uint32_t *level, uint32_t *out, uint32_t *d_out_count,
-                   uint32_t *tmp, uint32_t *scratch, cudaStream_t st);
 
 // Stable LSD radix sort of n pairs by key, over the 8-bit digits whose
 // indices are listed in `digits` (0 = least significant). keys/vals are

@@ -8,7 +8,7 @@ from paper_2412_18008_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
 
-LARGE = 1 << 14  # the smallest batch that uses labels (60 sqrt(n) at most for these sizes)
+LARGE = 1 << 14  # the smallest batch that uses labels (above 80 sqrt(n) for these sizes)
 
 
 def _ch():
