@@ -822,25 +822,30 @@ def main():
         # with stalling each expansion also reads the other CSR's two offsets
         stall = bool(qcfg[3]) if qcfg else False
         l2_record = None
-        if args.workload == "geo1M" and qcfg is not None and tuple(qcfg) == QUERY_L2_CONFIG:
+        # batches of this size, on a hierarchy without a core, are answered
+        # through hub labels (ch_query_batch), not by a search a query
+        labels = nq >= 1 << 14 and nq * nq >= 6400 * stats["n"] and not stats["core_vertices"]
+        if not labels and args.workload == "geo1M" and qcfg is not None and tuple(qcfg) == QUERY_L2_CONFIG:
             l2_peak = l2_read_gbs(dev)
             l2_gbs = QUERY_L2_BYTES_PER_QUERY * nq / (mean_query * 1e-3) / 1e9
             l2_record = {"bytes_per_query": QUERY_L2_BYTES_PER_QUERY, "achieved": round(l2_gbs, 1),
                          "peak": round(l2_peak, 1), "unit": "GB/s", "frac": round(l2_gbs / l2_peak, 4),
                          "peak_source": "measured: float32 sum over a 48 MB L2-resident buffer",
                          "bytes_source": "ncu lts__t_sectors of a 200K-query pass, per query"}
-        q_bytes = (20 if stall else 12) * q_exp + 8 * q_edges + 20 * nq
+        q_bytes = (0 if labels else (20 if stall else 12) * q_exp) + 8 * q_edges + 20 * nq
         q_gbs = q_bytes / (mean_query * 1e-3) / 1e9
         roofline = {
-            "kernel": "k_query_block (pruned bidirectional upward searches, one launch per batch)",
+            "kernel": ("k_hl_merge and k_hl_query (hub labels of the batch, then a join a query)" if labels else
+                       "k_query_block (pruned bidirectional upward searches, one launch per batch)"),
             "bound": "hbm", "achieved": round(q_gbs, 1), "peak": peak, "unit": "GB/s",
             "frac": round(q_gbs / peak, 4),
             # the captured traffic belongs to this workload in the default
             # configuration (warp layout, 256 threads, small tables, stalling)
-            "traffic": (QUERY_TRAFFIC_PER_LAUNCH if args.workload == "geo1M" and nq == 1_000_000
+            "traffic": (QUERY_TRAFFIC_PER_LAUNCH if not labels and args.workload == "geo1M" and nq == 1_000_000
                         and qcfg is not None and tuple(qcfg) == QUERY_L2_CONFIG else None),
             "peak_source": peak_src, "bytes_per_launch": q_bytes, "ms_per_launch": mean_query,
-            "launch": "one batch = the small-table pass + its overflow redo (two launches)",
+            "launch": ("one batch = a merge launch a level, the joins, and the searches of what had no label"
+                       if labels else "one batch = the small-table pass + its overflow redo (two launches)"),
             "expansions_per_query": q_exp / nq, "edges_per_query": q_edges / nq,
             "query_config": {"layout": ["block_flat", "warp_flat"][qcfg[0]] if qcfg else "default",
                              "threads": qcfg[1] if qcfg else None,
