@@ -2712,8 +2712,8 @@ struct Builder {
     uint32_t reads = 0;      // control blocks k_contract_prep has been asked for
     bool use_big = true;     // the middle tier's overflow goes to the big tier, not to the dense one
     // Phases left in which the big tier takes the middle tier's sources: set
-    // when a quarter of them outgrew the middle tier, whose attempts are then
-    // work done twice (16M-vertex geometric build: 2.50 -> 1.50 s).
+    // when five eighths of them outgrew the middle tier, whose attempts are then
+    // work done twice (16M-vertex geometric build: 2.50 -> 1.61 s; at a quarter 1.50, but RMAT 2^17 20.0 -> 24.6 ms).
     uint32_t skip_mid = 0;
     bool score_direct = false;  // the score phase skipped the warp tier
     // lists
@@ -3170,7 +3170,7 @@ void Builder::run_rounds() {
         if (skip_mid) {
             --skip_mid;  // the middle tier is tried again in the end
         } else {
-            if (use_big && nA && c.nOvf1 > 64 && 4ull * c.nOvf1 > (score_direct ? c.nS : c.nOvf)) skip_mid = 16;
+            if (use_big && nA && c.nOvf1 > 64 && 8ull * c.nOvf1 > 5ull * (score_direct ? c.nS : c.nOvf)) skip_mid = 16;
             use_big = (use_big ? c.nOvf1 : c.nOvf2) > 4;
         }
         if (nF == 0) {
