@@ -21,7 +21,11 @@ constexpr int QB_THREADS = 256;  // threads per query block, at most
 // direction (one bitmap per level parity, the idle one cleared during the
 // level), a double-buffered frontier holding both directions' entries
 // (slot | dir<<31), and a triple-buffered frontier counter and pair of
-// least queued labels (see block_search).
+// least queued labels (see block_search). A level that does not fit makes the
+// next one's count larger than FC: pushes past the frontier's end count on,
+// and a full table sets QB_FULL in it.
+constexpr uint32_t QB_FULL = 0x80000000u;
+
 template <int TB>
 struct QBSmem {
     static constexpr uint32_t T = 1u << TB;   // table slots
@@ -43,7 +47,7 @@ struct QBSmem {
     uint32_t wtot[QB_THREADS / 32 + 1];
     uint32_t cnt3[3];
     uint32_t lmin3[3][2];  // least label queued per level (mod 3) and direction
-    uint32_t item, ovf, mu, cnt, ss, st;
+    uint32_t item, mu, cnt;
 };
 
 struct QArgs {
@@ -135,7 +139,8 @@ struct QStat {
 };
 
 // Relaxes one edge e = (y, w) of a vertex labelled dx in direction dir.
-// Returns nothing; records an overflow in q.ovf, an index error in a.err.
+// Returns nothing; records an overflow in the next level's count, an index
+// error in a.err.
 // With TRACK, lmf / lmb keep the least new forward / backward label this
 // thread has set in the level (every vertex whose label drops is queued for
 // the next level).
@@ -152,7 +157,7 @@ __device__ __forceinline__ void qb_relax(QBSmem<TB> &q, const QArgs &a, uint32_t
     if (PRUNE && nd >= q.mu) return;
     const uint32_t ys = qb_insert<TB>(q.key, e.x);
     if (ys == EMPTY) {
-        q.ovf = 1;
+        atomicOr(&q.cnt3[nxt_cnt], QB_FULL);
         return;
     }
     uint32_t *dist = dir ? q.db : q.df;
@@ -169,7 +174,6 @@ __device__ __forceinline__ void qb_relax(QBSmem<TB> &q, const QArgs &a, uint32_t
     if (qb_claim(q, ys, dir, lvl)) {
         const uint32_t p = atomicAdd(&q.cnt3[nxt_cnt], 1u);
         if (p < QBSmem<TB>::FC) next_front[p] = ys | (dir << 31);
-        else q.ovf = 1;
     }
 }
 
@@ -259,10 +263,14 @@ __device__ __forceinline__ void qb_entry_both(const QBSmem<TB> &q, const QArgs &
 // Barrier discipline: the frontier counter of level k lives in cnt3[k % 3],
 // and (DELTA) the least labels queued for it in lmin3[k % 3]; thread 0
 // clears both for level k + 2 during level k, when no thread reads them any
-// more. Each level reads its frontier size and the overflow
-// flag right after a barrier that follows every write to them: the barrier
-// at the top of the level (warp-flattened; block-flattened at level 1) or
-// the barrier that ends the previous level's last tile (block-flattened).
+// more. Each level reads its frontier size, which also says that the level
+// before overflowed, right after a barrier that follows every write to it: the
+// barrier at the top of the level (warp-flattened; block-flattened at level 1)
+// or the barrier that ends the previous level's last tile (block-flattened).
+// Nothing that a level writes is read at its own top, so every warp leaves the
+// search at the same barrier. (One overflow flag for all levels would not do:
+// a warp late at a level's top would see it set by a warp already in that
+// level, leave one level early and stay a barrier ahead of the block.)
 template <bool PRUNE, bool WARP, int TB, bool STALL, bool DELTA = false>
 __device__ bool block_search(QBSmem<TB> &q, const QArgs &a, QStat &stat) {
     static_assert(!DELTA || (PRUNE && WARP), "delta-stepping levels: pruned warp-flattened searches");
@@ -273,8 +281,7 @@ __device__ bool block_search(QBSmem<TB> &q, const QArgs &a, QStat &stat) {
         if (WARP || lvl == 1) __syncthreads();
         const uint32_t cur = (lvl - 1) & 1u;
         const uint32_t nfront = q.cnt3[(lvl - 1) % 3];
-        const uint32_t ovf = q.ovf;
-        if (ovf) return false;
+        if (nfront > FC) return false;
         if (nfront == 0) return true;
         if (lvl >= 0xFFFFu) {  // a label-correcting search on a DAG never gets here
             if (tid == 0) atomicOr(a.err, QERR_BOUND);
@@ -319,7 +326,6 @@ __device__ bool block_search(QBSmem<TB> &q, const QArgs &a, QStat &stat) {
                         p = __shfl_sync(FULL, p, leader) + __popc(m & ((1u << lane) - 1u));
                         if (won) {
                             if (p < FC) next_front[p] = ent;
-                            else q.ovf = 1;
                             if (edir) lmb = min(lmb, lab);
                             else lmf = min(lmf, lab);
                         }
@@ -475,7 +481,6 @@ __device__ bool block_query_by(QBSmem<TB> &q, const QArgs &a, uint32_t rs, uint3
         q.df[ss] = 0;
         const uint32_t st = qb_insert<TB>(q.key, rt);
         q.db[st] = 0;
-        q.ovf = 0;
         q.mu = ss == st ? 0u : INF;
         q.cnt = 0;
         q.front[0][0] = ss;

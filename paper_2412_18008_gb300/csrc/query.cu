@@ -393,8 +393,7 @@ __device__ bool row_search(QBSmem<TB> &q, const QArgs &a, QStat &stat) {
         __syncthreads();
         const uint32_t cur = (lvl - 1) & 1u;
         const uint32_t nfront = q.cnt3[(lvl - 1) % 3];
-        const uint32_t ovf = q.ovf;
-        if (ovf) return false;
+        if (nfront > FC) return false;
         if (nfront == 0) return true;
         if (lvl >= 0xFFFFu) {
             if (tid == 0) atomicOr(a.err, QERR_BOUND);
@@ -423,7 +422,6 @@ __device__ bool row_search(QBSmem<TB> &q, const QArgs &a, QStat &stat) {
                 if (qb_claim(q, slot, dir, lvl)) {
                     const uint32_t p = atomicAdd(&q.cnt3[nxt_cnt], 1u);
                     if (p < FC) next_front[p] = ent;
-                    else q.ovf = 1;
                     if (dir) lmb = min(lmb, lab);
                     else lmf = min(lmf, lab);
                 }

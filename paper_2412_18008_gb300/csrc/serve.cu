@@ -161,10 +161,10 @@ __device__ __forceinline__ bool sv_claim(uint32_t *fst, uint32_t slot, uint32_t 
 
 // Fallback for a pair whose search spaces overflow the shared table: the
 // same search (warp-flattened levels, no stalling), labels in the block's
-// global hash table. Control values (s_cnt3, s_ovf) are read between two
-// barriers as in block_search. Returns INF when unreachable.
+// global hash table. Control values are read as in block_search, the overflow
+// again with the level's count. Returns INF when unreachable.
 __device__ uint32_t sv_query(const SvArgs &a, const Tab &t, uint32_t rs, uint32_t rt,
-                             uint32_t *s_cnt3, uint32_t *s_ovf, uint32_t *s_mu, uint32_t *s_nt) {
+                             uint32_t *s_cnt3, uint32_t *s_mu, uint32_t *s_nt) {
     const QArgs &g = a.q;
     const uint32_t tid = threadIdx.x;
     __syncthreads();
@@ -179,15 +179,15 @@ __device__ uint32_t sv_query(const SvArgs &a, const Tab &t, uint32_t rs, uint32_
         s_cnt3[0] = 2;
         s_cnt3[1] = 0;
         s_cnt3[2] = 0;
-        *s_ovf = 0;
         *s_mu = ss == st ? 0u : INF;
     }
+    bool full = false;
     for (uint32_t lvl = 1;; ++lvl) {
         __syncthreads();
         const uint32_t cur = (lvl - 1) & 1u;
         const uint32_t nfront = s_cnt3[(lvl - 1) % 3];
-        const uint32_t ovf = *s_ovf;
-        if (ovf || nfront == 0 || lvl >= 0xFFFFu) break;
+        full = nfront > t.fcap;
+        if (full || nfront == 0 || lvl >= 0xFFFFu) break;
         if (tid == 0) s_cnt3[(lvl + 1) % 3] = 0;
         const uint32_t *fr = t.front + (size_t)cur * t.fcap;
         uint32_t *fn = t.front + (size_t)(cur ^ 1u) * t.fcap;
@@ -238,7 +238,7 @@ __device__ uint32_t sv_query(const SvArgs &a, const Tab &t, uint32_t rs, uint32_
                 if (nd == INF || nd >= *(volatile uint32_t *)s_mu) continue;
                 const uint32_t ys = sv_insert(t, e.x, a.tbits, s_nt);
                 if (ys == EMPTY) {
-                    *s_ovf = 1;
+                    atomicOr(&s_cnt3[lvl % 3], QB_FULL);
                     continue;
                 }
                 uint32_t *dist = odir ? t.db : t.df;
@@ -249,13 +249,12 @@ __device__ uint32_t sv_query(const SvArgs &a, const Tab &t, uint32_t rs, uint32_
                 if (sv_claim(t.fst, ys, odir, lvl)) {
                     const uint32_t p = atomicAdd(&s_cnt3[lvl % 3], 1u);
                     if (p < t.fcap) fn[p] = ys | (odir << 31);
-                    else *s_ovf = 1;
                 }
             }
         }
     }
     __syncthreads();
-    if (*s_ovf && tid == 0) atomicOr(a.status, QERR_BOUND);
+    if (full && tid == 0) atomicOr(a.status, QERR_BOUND);
     // the answer: least meeting sum over the reached vertices
     const uint32_t nt = *s_nt;
     uint32_t mu = INF;
@@ -428,7 +427,7 @@ __global__ void __launch_bounds__(QB_THREADS, TB == 11 ? 6 : 1) k_serve(SvArgs a
             if (rs < g.n && rt < g.n) {
                 uint32_t cnt;
                 if (!block_query<true, WARP, TB, STALL, DELTA>(q, g, rs, rt, ans, cnt, stat))
-                    ans = sv_query(a, t, rs, rt, q.cnt3, &q.ovf, &q.mu, &q.cnt);
+                    ans = sv_query(a, t, rs, rt, q.cnt3, &q.mu, &q.cnt);
             } else if (tid == 0) {
                 atomicOr(a.status, QERR_BOUND);
             }
