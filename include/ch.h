@@ -265,8 +265,9 @@ int ch_query_batch_host(ch_t *ch, const uint32_t *src, const uint32_t *dst, uint
  * until the process exits. The first call on a device resolves that array's
  * device address (cudaGetSymbolAddress) with the device current, so make
  * the first call on each device before any stream capture. All calls on a
- * device share the array (every call's last kernel leaves its counters at
- * zero): calls whose work overlaps on the GPU race on it, so serialise them (one stream, or events), across handles too.
+ * device share the array, which keeps the last call's contents (the call
+ * clears the counters it needs): calls whose work overlaps on the GPU race
+ * on it, so serialise them (one stream, or events), across handles too.
  * The hierarchy's device must be the current device (the scratch address is
  * resolved per current device). Errors: CH_ERANGE when
  * k > CH_STATIC_QUERY_MAX; CH_EINVAL when another device is current; ids >= n

@@ -64,11 +64,13 @@ struct QArgs {
     // query j for j < k, or, with in_list, query in_list[j] for
     // j < work[in_cnt]. A query whose search overflows is appended to ovf,
     // counted in work[ovf_cnt]. The dense kernel takes ovf entries (or, with
-    // dense_first, all queries) from work[1].
+    // dense_first, all queries) from work[1]. With ovf_flags (small batches)
+    // there are no counters: ovf[j] says whether query j overflowed.
     uint32_t *work;
     const uint32_t *in_list;
-    uint32_t in_cnt, ctr, ovf_cnt, ticket;  // (ticket: the dense kernel's finished blocks, the last counter)
+    uint32_t in_cnt, ctr, ovf_cnt;
     uint32_t *ovf;
+    bool ovf_flags = false;
     uint32_t *err;
     unsigned long long *stats;  // [0] expansions, [1] edges scanned (or null)
     // Core distance table (or null): the searches do not expand the core's

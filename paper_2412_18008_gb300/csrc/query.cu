@@ -27,8 +27,8 @@ namespace gbch {
 namespace {
 
 constexpr uint64_t Q_CHUNK = 1u << 22;  // queries per launch pair
-// Counters of a batch: zero between batches (its last kernel, the dense one,
-// clears them), the last one counts that kernel's finished blocks.
+// Counters of a batch, cleared at its start: what an earlier batch left behind,
+// whole or not, does not matter to the next. (Small batches have none.)
 constexpr uint32_t QWORK = 8;
 
 // (The stalling variants are held to six resident blocks per SM, about 40
@@ -340,14 +340,24 @@ __global__ void __launch_bounds__(QD_THREADS) k_query_dense(QArgs a, QDense dn) 
     __shared__ QDSmem q;
     const uint32_t tid = threadIdx.x;
     pdl_wait();
-    const uint32_t nitems = a.dense_first ? (uint32_t)a.k : a.work[a.ovf_cnt];
+    const uint32_t nitems = a.ovf_flags || a.dense_first ? (uint32_t)a.k : a.work[a.ovf_cnt];
     QStat stat;
-    while (nitems) {
-        __syncthreads();
-        if (tid == 0) q.item = atomicAdd(&a.work[1], 1u);
-        __syncthreads();
-        if (q.item >= nitems) break;
-        const uint32_t i = a.dense_first ? q.item : a.ovf[q.item];
+    bool worked = false;
+    for (uint32_t next = blockIdx.x; nitems;) {
+        uint32_t i;
+        if (a.ovf_flags) {
+            if (next >= nitems) break;
+            i = next;
+            next += gridDim.x;
+            if (!a.ovf[i]) continue;
+        } else {
+            __syncthreads();
+            if (tid == 0) q.item = atomicAdd(&a.work[1], 1u);
+            __syncthreads();
+            if (q.item >= nitems) break;
+            i = a.dense_first ? q.item : a.ovf[q.item];
+        }
+        worked = true;
         if (i >= a.k) {
             if (tid == 0) atomicOr(a.err, QERR_BOUND);
             continue;
@@ -360,17 +370,12 @@ __global__ void __launch_bounds__(QD_THREADS) k_query_dense(QArgs a, QDense dn) 
             if (a.settled) a.settled[i] = cnt;
         }
     }
-    if (nitems) qb_flush_stat(stat, a.stats);
-    // The last block to finish leaves the batch's counters at zero for the
-    // next batch. (Every block has read the overflow count before it counts
-    // itself finished.)
-    __syncthreads();
-    if (tid == 0 && atomicAdd(&a.work[a.ticket], 1u) + 1 == gridDim.x)
-        for (uint32_t w = 0; w <= a.ticket; ++w) a.work[w] = 0;
+    if (worked) qb_flush_stat(stat, a.stats);
 }
 
 // Small batches: a block of 1024 threads a query, in one launch; queries that
-// outgrow the table are left to the dense kernel behind it. With that few
+// outgrow the table are flagged for the dense kernel behind it (a flag a query
+// in place of a list, so that there is no counter to clear). With that few
 // queries the time of one counts: the chain of round trips of its levels, and
 // how fast one SM issues their instructions. The levels are block_search's,
 // with stalling and buckets, but a warp takes whole rows: a level's entries
@@ -473,12 +478,12 @@ __global__ void __launch_bounds__(QS_THREADS, 1) k_query_small(QArgs a) {
     qb_clear(q);
     for (uint32_t i = blockIdx.x; i < a.k; i += gridDim.x) {
         uint32_t rs, rt, mu, cnt;
-        if (!query_ranks(a, i, rs, rt)) continue;
-        if (!block_query_by(q, a, rs, rt, mu, cnt, [&] { return row_search<12>(q, a, stat); })) {
-            if (threadIdx.x == 0) a.ovf[atomicAdd(&a.work[a.ovf_cnt], 1u)] = i;
-            continue;
+        bool ok = true;
+        if (query_ranks(a, i, rs, rt)) {
+            ok = block_query_by(q, a, rs, rt, mu, cnt, [&] { return row_search<12>(q, a, stat); });
+            if (threadIdx.x == 0 && ok) a.out[i] = mu;
         }
-        if (threadIdx.x == 0) a.out[i] = mu;
+        if (threadIdx.x == 0) a.ovf[i] = !ok;
     }
     qb_flush_stat(stat, a.stats);
 }
@@ -574,7 +579,6 @@ void query_init(ch_s *h) {
     h->qerr.alloc(1);
     h->qerr.zero(0);
     h->qwork.alloc(QWORK);
-    h->qwork.zero(0);
     h->q_ovf_cap = Q_CHUNK;
     h->q_ovf_list.alloc(2 * Q_CHUNK);  // overflow lists of the two block-kernel passes
     // as many slots as the chip runs blocks of the dense kernel at once (two
@@ -673,9 +677,12 @@ namespace {
 // vertices: 126 and 120 us). Not for queries that need the dense kernel.
 bool small_batch(const QArgs &a, uint64_t k) { return k <= (uint64_t)device_sm_count() && !a.dense_first; }
 
-void launch_query_small(const QArgs &a, cudaStream_t st) {
+// (a.ovf: room for k flags)
+void launch_query_small(const ch_s *h, QArgs &a, cudaStream_t st) {
+    a.ovf_flags = true;
     k_query_small<<<(unsigned)a.k, QS_THREADS, sizeof(QBSmem<12>), st>>>(a);
     CH_CHECK_LAUNCH();
+    launch_query_dense(h, a, true, a.k, st);
 }
 
 }  // namespace
@@ -690,12 +697,8 @@ bool query_batch_small(ch_s *h, const uint32_t *src, uint32_t one_src, const uin
     a.out = dist_out;
     a.settled = nullptr;
     a.k = k;
-    a.work = h->qwork.ptr;
-    a.ticket = QWORK - 1;
     a.ovf = h->q_ovf_list.ptr;
-    a.ovf_cnt = 2;
-    launch_query_small(a, st);
-    launch_query_dense(h, a, true, k, st);
+    launch_query_small(h, a, st);
     return true;
 }
 
@@ -712,9 +715,9 @@ void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
         a.settled = settled_out ? settled_out + c0 : nullptr;
         a.k = kc;
         a.work = h->qwork.ptr;
-        a.ticket = QWORK - 1;
         a.in_list = nullptr;
         a.in_cnt = 0;
+        CH_CUDA_TRY(cudaMemsetAsync(a.work, 0, QWORK * sizeof(uint32_t), st));
         // Pruned searches unless the caller asked for search-space sizes,
         // which are defined by the exhaustive upward searches.
         const bool prune = settled_out == nullptr;
@@ -972,7 +975,7 @@ void query_graph_free(ch_query_graph_s *g) {
 
 namespace {
 
-constexpr uint32_t kStaticScratchHead = 4;  // [0] block counter, [1] dense counter, [2] overflow count, [3] finished blocks
+constexpr uint32_t kStaticScratchHead = 4;  // [0] block counter, [1] dense counter, [2] overflow count
 __device__ __align__(256) uint32_t g_static_query_scratch[kStaticScratchHead + CH_STATIC_QUERY_MAX];
 
 std::mutex g_static_mu;
@@ -1018,10 +1021,11 @@ void query_batch_static(ch_s *h, const uint32_t *src, const uint32_t *dst, uint6
     a.ctr = 0;
     a.ovf = scratch + kStaticScratchHead;
     a.ovf_cnt = 2;
-    a.ticket = kStaticScratchHead - 1;
+    if (small_batch(a, k)) return launch_query_small(h, a, st);
+    // the counters keep the previous call's values: clear them
+    CH_CUDA_TRY(cudaMemsetAsync(scratch, 0, kStaticScratchHead * sizeof(uint32_t), st));
     // one block-kernel pass (large tables): the scratch holds one list
-    if (small_batch(a, k)) launch_query_small(a, st);
-    else if (!a.dense_first) launch_query_block(h, a, true, false, k, st);
+    if (!a.dense_first) launch_query_block(h, a, true, false, k, st);
     launch_query_dense(h, a, true, k, st);
 }
 
