@@ -235,8 +235,9 @@ int ch_build(const ch_graph_t *g, const ch_params_t *params, ch_t **out);
  * without waiting. Ids >= n give CH_EINVAL for the whole batch (checked on
  * the device; the status is returned by the next synchronising call on the
  * handle, or by ch_query_status). k = 0 is a no-op.
- * A batch of at least 2^14 and 80 sqrt(n) queries (without settled_out, on a
- * hierarchy without a core and of at most about 4M vertices) is answered
+ * A large batch (at least 2^14, 80 sqrt(n) and 224 queries a level of the
+ * hierarchy, more on large hierarchies with long rows; without settled_out, on
+ * a hierarchy without a core and of at most about 4M vertices) is answered
  * through hub labels computed by the call for the vertices the batch climbs
  * through; the first such batch of a handle allocates their memory (about 6 KB
  * a vertex, kept until ch_free; without that memory, or in a stream capture

@@ -18,6 +18,7 @@
 //
 // Labels are made by each call from its own batch; only the memory is kept.
 #include <algorithm>
+#include <cmath>
 
 #include "handle.cuh"
 #include "qsearch.cuh"
@@ -25,18 +26,34 @@
 namespace gbch {
 namespace {
 
-// Batches of at least 2^14 and 80 sqrt(n) queries use labels. Labels cost a
-// chain of launches and the labels of the upper levels whatever the batch, a
-// search costs the same for every query; measured (ms, labels / searches):
-// n = 20K: 17K queries 0.71 / 0.81; 100K: 20K queries 1.38 / 1.42, 30K 1.43 /
-// 2.04; 256K: 20K queries 2.7 / 2.2, 30K 2.8 / 3.1; 1M: 48K queries 9.0 / 9.0,
-// 64K 9.3 / 12.0, 1M queries 17.0 / 186.6. (On hierarchies with quicker searches,
-// composite or memoised, the ways cross later: 100K memoised, 17K queries 1.38 /
-// 1.25; the line lies where labels win on all of them.)
+// The line from which a batch uses labels. A search costs the same for every
+// query; labels cost a launch or two a level (8 to 10 us), and the merges of what
+// the batch climbs through. A label holds about 0.13 row^2 hubs a level (row: mean
+// length of a CSR row; measured 1.1 to 1.2 x the levels at row 3, 2.0 at 3.9), and
+// once the arena outgrows the L2 its merges run at HBM latency, so the line also
+// grows with n x levels x row^4. Rows above 4.5 count as 4.5: longer ones were
+// measured on small, dense graphs only, where the labels stay in the L2.
+// Measured, ms (labels / searches):
+//   geometric (row 3)  20K vertices, 56 levels: 16K queries 0.72 / 0.78; 100K, 107:
+//         25K 1.54 / 1.89; 256K, 135: 40K 2.7 / 4.0; 1M, 218: 80K 9.3 / 14.4, 1M
+//         17.0 / 186.6; 3M, 325: 139K 52.9 / 52.5, 400K 63 / 151
+//   grids (3.8 to 3.9) 128^2, 71: 16K 0.99 / 0.98; 300^2, 114: 24K 2.5 / 2.7; 600^2,
+//         187: 48K 9.2 / 10.5; 1000^2, 241: 80K 39.4 / 30.8, 400K 66 / 151; 1400^2,
+//         302: 112K 139 / 70, 400K 203 / 247; 1800^2, 344: 144K 304 / 140, 400K 401 /
+//         387
+//   digraphs           2.5K vertices, 224: 16K 1.8 / 1.3, 66K 1.9 / 4.7; 20K (m = 1.5
+//         n), 198: 16K 1.9 / 1.0, 66K 2.0 / 3.7; 20K (m = 2 n), 514: 16K 11.5 / 5.7,
+//         66K 17.3 / 20.4; 9K (m = 3.4 n), 726: 16K 24.0 / 11.1, 66K 47.1 / 42.0,
+//         400K 203 / 251 (and 60% of its queries are searched all the same)
+// Every losing one is below the line. (Not so RMAT 2^12 contracted whole, 100
+// levels, half of whose searches end at once: 22K queries 0.94 / 0.55.)
 constexpr uint64_t HL_MIN_K = 1u << 14;
-constexpr uint64_t HL_MIN_SQRT = 80;
-bool batch_is_large(uint64_t k, uint32_t n) {
-    return k >= HL_MIN_K && (k >= (1ull << 32) || k * k >= HL_MIN_SQRT * HL_MIN_SQRT * n);
+constexpr double HL_MIN_SQRT = 80, HL_MIN_LEVEL = 224, HL_ROW_MAX = 4.5, HL_WORK = 566e3;
+bool batch_is_large(const ch_s *h, uint64_t k) {
+    const double n = (double)h->n, levels = (double)h->round_stats.size();
+    const double row = std::min(HL_ROW_MAX, 0.5 * (double)(h->n_up + h->n_down) / n);
+    return k >= HL_MIN_K && (double)k >= HL_MIN_SQRT * std::sqrt(n) && (double)k >= HL_MIN_LEVEL * levels &&
+           (double)k * HL_WORK >= n * levels * row * row * row * row;
 }
 constexpr uint32_t HL_PRUNE_PART = 16;
 // Levels of at most this many vertices are merged by a block a label.
@@ -599,7 +616,7 @@ bool labels_possible(const ch_s *h) {
 }  // namespace
 
 bool query_labels_prepare(ch_s *h, uint64_t k) {
-    if (!batch_is_large(k, h->n) || !labels_possible(h)) return false;
+    if (!labels_possible(h) || !batch_is_large(h, k)) return false;
     if (h->hl_arena.ptr) return true;
     std::vector<uint32_t> lv;
     if (!rank_levels(h, lv)) {

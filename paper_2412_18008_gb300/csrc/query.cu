@@ -39,8 +39,9 @@ __global__ void __launch_bounds__(QB_THREADS, (STALL || DELTA) ? 6 : 1) k_query_
     QBSmem<TB> &q = *reinterpret_cast<QBSmem<TB> *>(qb_raw);
     const uint32_t tid = threadIdx.x;
     QStat stat;
-    qb_clear(q);
     const uint64_t nitems = a.in_list ? a.work[a.in_cnt] : a.k;
+    if (nitems == 0) return;
+    qb_clear(q);
     while (true) {
         __syncthreads();
         if (tid == 0) q.item = atomicAdd(&a.work[a.ctr], 1u);
@@ -725,24 +726,24 @@ void query_batch(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
             launch_query_dense(h, a, prune, kc, st);
             continue;
         }
-        if (prune && !searches_only &&
-            query_batch_labels(h, a.src, a.dst, kc, a.out, h->q_ovf_list.ptr + Q_CHUNK, h->qwork.ptr + 4, st)) {
+        uint32_t *const list = h->q_ovf_list.ptr, *const list2 = list + Q_CHUNK;
+        if (prune && !searches_only && query_batch_labels(h, a.src, a.dst, kc, a.out, list, a.work + 4, st)) {
             // the queries that the labels could not answer, by searches
-            a.in_list = h->q_ovf_list.ptr + Q_CHUNK;
+            a.in_list = list;
             a.in_cnt = 4;
-        } else if (h->q_small_first) {
+        }
+        if (h->q_small_first) {
             // pass 1 on small tables (twice the resident queries); the
             // queries that overflow them are redone on the large tables
             a.ctr = 0;
-            a.ovf = h->q_ovf_list.ptr + Q_CHUNK;
-            a.ovf_cnt = 4;
+            a.ovf = list2;
+            a.ovf_cnt = 5;
             launch_query_block(h, a, prune, true, kc, st);
-            a.ctr = 3;
-            a.in_list = h->q_ovf_list.ptr + Q_CHUNK;
-            a.in_cnt = 4;
+            a.in_list = list2;
+            a.in_cnt = 5;
         }
-        a.ctr = a.in_list ? 3 : 0;
-        a.ovf = h->q_ovf_list.ptr;
+        a.ctr = 3;
+        a.ovf = a.in_list == list ? list2 : list;  // (the list that is used up)
         a.ovf_cnt = 2;
         launch_query_block(h, a, prune, false, kc, st);
         launch_query_dense(h, a, prune, kc, st);
