@@ -519,7 +519,11 @@ int ch_mlp_forward(const float *weights, const int64_t *rows, uint64_t n, float 
  * after it has ended at the idle limit; keep them out of serving windows or
  * choose a short idle_ms. The handle `ch` must outlive the server. */
 typedef struct {
-    uint32_t blocks;   /* blocks of the device loop; 0 = as many as are resident at once */
+    uint32_t blocks;   /* blocks of the device loop; 0 = as many as are resident at once: six
+                        * an SM for hierarchies of up to 400,000 vertices whose searches fit
+                        * 2^11-slot tables (the first server of a handle tries 512), else
+                        * three. Each holds up to 4.7 MB of device memory (36 B a vertex up
+                        * to 2^17); short of memory for six an SM, three are run */
     uint32_t ring;     /* requests in flight at most */
     uint64_t pool;     /* target/answer entries at most */
     uint32_t idle_ms;  /* idle limit of the device loop */

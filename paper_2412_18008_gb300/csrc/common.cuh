@@ -27,6 +27,10 @@ struct Error {
     std::string msg;
 };
 
+// Whether e is a real lack of memory, which a caller may answer with a way that
+// needs less (an injected failure is the library's caller's to see).
+inline bool out_of_memory(const Error &e) { return e.code == CH_ENOMEM && e.msg.rfind("injected", 0) != 0; }
+
 void set_last_error(const char *fmt, ...);
 
 #define CH_CUDA_TRY(expr)                                                        \

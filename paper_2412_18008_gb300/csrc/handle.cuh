@@ -68,6 +68,7 @@ struct ch_s {
     uint32_t q_stall = 1;        // stall on demand (warp layout, pruned searches)
     uint32_t q_delta = 0;        // delta-stepping bucket width (warp layout; 0: off)
     uint32_t q_wscale = 1;       // weight scale: median of sampled E_up weights
+    int q_fits_small = -1;       // query_fits_small's answer for this configuration; -1: not sampled yet
     uint32_t q_slots = 0;
     uint64_t q_ovf_cap = 0;
     gbch::DevBuf<uint32_t> q_src_fill;  // repeated source of one-to-many queries
@@ -133,6 +134,9 @@ void query_set_config(ch_s *h, uint32_t layout, uint32_t threads, uint32_t small
 void query_autotune(ch_s *h, uint64_t sample, uint32_t seed, cudaStream_t st, ch_query_config_t *chosen,
                     double *ms_out);
 void query_work(ch_s *h, cudaStream_t st, uint64_t out[2]);
+// Whether nearly all searches of the handle's configuration fit 2^11-slot tables
+// (a sample of seeded random pairs, run on `st` and waited for the first time).
+bool query_fits_small(ch_s *h, cudaStream_t st);
 // Device time (ms) of a batch of `sample` seeded random queries (after one warm-up batch).
 double query_time_sample(ch_s *h, uint64_t sample, uint32_t seed, cudaStream_t st);
 ch_query_graph_s *query_graph_create(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,

@@ -643,9 +643,8 @@ bool query_labels_prepare(ch_s *h, uint64_t k) {
         h->hl_cursor = std::move(cursor);
         h->hl_arena = std::move(arena);
     } catch (const Error &e) {
-        // no memory for labels: the searches need none of it (an injected
-        // failure is the caller's to see)
-        if (e.code != CH_ENOMEM || e.msg.rfind("injected", 0) == 0) throw;
+        // no memory for labels: the searches need none of it
+        if (!out_of_memory(e)) throw;
         h->hl_off = true;
         return false;
     }

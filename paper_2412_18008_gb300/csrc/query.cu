@@ -783,6 +783,39 @@ void query_set_config(ch_s *h, uint32_t layout, uint32_t threads, uint32_t small
     h->q_small_first = small_first;
     h->q_stall = stall;
     h->q_delta = delta;
+    h->q_fits_small = -1;
+}
+
+bool query_fits_small(ch_s *h, cudaStream_t st) {
+    constexpr uint32_t SAMPLE = 512, MOST = SAMPLE / 32;  // (see server_start for the line)
+    if (h->q_fits_small >= 0) return h->q_fits_small;
+    if (h->n == 0) return true;
+    // buffers of its own: a batch may be in flight on another stream
+    DevBuf<uint32_t> buf;
+    buf.alloc(QWORK + 4 * SAMPLE);
+    CH_CUDA_TRY(cudaMemsetAsync(buf.ptr, 0, QWORK * sizeof(uint32_t), st));
+    uint32_t *s = buf.ptr + QWORK, *t = s + SAMPLE;
+    k_sample_pairs<<<(SAMPLE + 255) / 256, 256, 0, st>>>(s, t, SAMPLE, h->n, 1u);
+    CH_CHECK_LAUNCH();
+    QArgs a = hierarchy_args(h);
+    a.core_tab = nullptr;  // (the server's searches do not use it)
+    a.stats = nullptr;
+    a.settled = nullptr;
+    a.src = s;
+    a.dst = t;
+    a.out = t + SAMPLE;
+    a.k = SAMPLE;
+    a.work = buf.ptr;
+    a.in_list = nullptr;
+    a.ctr = 0;
+    a.ovf = a.out + SAMPLE;
+    a.ovf_cnt = 2;
+    launch_query_block(h, a, true, true, SAMPLE, st);
+    uint32_t over = 0;
+    CH_CUDA_TRY(cudaMemcpyAsync(&over, a.work + a.ovf_cnt, sizeof over, cudaMemcpyDeviceToHost, st));
+    CH_CUDA_TRY(cudaStreamSynchronize(st));
+    h->q_fits_small = over <= MOST;
+    return h->q_fits_small;
 }
 
 void query_autotune(ch_s *h, uint64_t sample, uint32_t seed, cudaStream_t st, ch_query_config_t *chosen,

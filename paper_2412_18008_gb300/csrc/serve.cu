@@ -537,21 +537,28 @@ void server_start(ch_server_s *sv, ch_s *h, const ch_server_params_t *p) {
     // the handle's query configuration (layout and block size)
     const bool warp = h->q_layout == CH_QUERY_WARP_FLAT;
     const int threads = (int)h->q_threads;
-    // The searches of hierarchies of up to SV_SMALL_N vertices fit 2^11-slot
-    // tables, which put six blocks on an SM instead of three (256K vertices, a
-    // burst of 80,000 pairs: 26.9 -> 11.1 ms, SV_TAKE included). Larger ones
-    // keep 2^12: a pair that overflows is redone on the block's slower global
-    // table.
-    const bool small = warp && h->q_stall && h->q_delta && h->n <= SV_SMALL_N;
-    auto kern = warp ? (h->q_stall ? (h->q_delta ? (small ? k_serve<true, true, true, 11> : k_serve<true, true, true>)
-                                                 : k_serve<true, true>)
-                                   : k_serve<true, false>)
-                     : k_serve<false, false>;
-    sv->smem = small ? sizeof(QBSmem<11>) : sizeof(QBSmem<12>);
-    CH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv->smem));
-    int per_sm = 0;
-    CH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sv->smem));
-    sv->nblocks = p->blocks ? p->blocks : (uint32_t)sms * (uint32_t)std::max(per_sm, 1);
+    CH_CUDA_TRY(cudaStreamCreateWithFlags(&sv->st, cudaStreamNonBlocking));
+    void (*kern)(SvArgs) = nullptr;
+    auto configure = [&](bool small) {
+        kern = warp ? (h->q_stall ? (h->q_delta ? (small ? k_serve<true, true, true, 11> : k_serve<true, true, true>)
+                                                : k_serve<true, true>)
+                                  : k_serve<true, false>)
+                    : k_serve<false, false>;
+        sv->smem = small ? sizeof(QBSmem<11>) : sizeof(QBSmem<12>);
+        CH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv->smem));
+        int per_sm = 0;
+        CH_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sv->smem));
+        sv->nblocks = p->blocks ? p->blocks : (uint32_t)sms * (uint32_t)std::max(per_sm, 1);
+    };
+    // 2^11-slot tables put six blocks on an SM instead of three, but a pair that
+    // overflows them is redone on the block's slower global table: they serve
+    // hierarchies of up to SV_SMALL_N vertices at most one in 32 of whose sampled
+    // searches overflow. A burst of 40,000 pairs, 2^11 / 2^12 slots: geometric,
+    // none overflow, 256K vertices 6.4 / 7.2 ms, 400K 6.7 / 8.2; grid of 600 x 600,
+    // none, 10.0 / 13.2; digraphs, one in 10, 17.0 / 17.9 and a p99 service time of
+    // 3.8 / 1.3; four in 10, 38.0 / 28.4 and 7.7 / 2.2.
+    bool small = warp && h->q_stall && h->q_delta && h->n <= SV_SMALL_N && query_fits_small(h, sv->st);
+    configure(small);
     uint32_t tbits = 10;
     while (tbits < 24 && ((1u << tbits) < std::min<uint32_t>(h->n, 1u << 17))) ++tbits;
     const size_t T = (size_t)1 << tbits;
@@ -569,10 +576,18 @@ void server_start(ch_server_s *sv, ch_s *h, const ch_server_params_t *p) {
     sv->consumed.assign(sv->ring, 0);
     // per block: key, df, db, fst, touched (T each) and two frontiers (fcap each)
     const size_t per_block = 5 * T + 2 * fcap;
-    sv->scratch.alloc(per_block * sv->nblocks);
+    const uint32_t more = sv->nblocks;
+    try {
+        sv->scratch.alloc(per_block * more);
+    } catch (const Error &e) {
+        // twice the blocks need twice the scratch: without it, fewer of them
+        if (!small || !out_of_memory(e)) throw;
+        configure(false);
+        if (sv->nblocks >= more) throw;
+        sv->scratch.alloc(per_block * sv->nblocks);
+    }
     uint32_t *base = sv->scratch.ptr;
     const size_t NB = sv->nblocks;
-    CH_CUDA_TRY(cudaStreamCreateWithFlags(&sv->st, cudaStreamNonBlocking));
     CH_CUDA_TRY(cudaMemsetAsync(base, 0xFF, 3 * T * NB * 4, sv->st));           // key, df, db
     CH_CUDA_TRY(cudaMemsetAsync(base + 3 * T * NB, 0, T * NB * 4, sv->st));      // fst
     sv->claimed.alloc(1);
