@@ -239,9 +239,11 @@ int ch_build(const ch_graph_t *g, const ch_params_t *params, ch_t **out);
  * hierarchy, more on large hierarchies with long rows; without settled_out, on
  * a hierarchy without a core and of at most about 4M vertices) is answered
  * through hub labels computed by the call for the vertices the batch climbs
- * through; the first such batch of a handle allocates their memory (about 6 KB
- * a vertex, kept until ch_free; without that memory, or in a stream capture
- * before it exists, the batch is searched query by query). Same answers. */
+ * through. The first such batch of a handle allocates their memory, about 6 KB a
+ * vertex, if that is at most a quarter of what the device has free. It is kept
+ * until ch_free, and like all of a hierarchy's memory then stays in the
+ * library's cache until ch_trim_memory. Without it, or in a stream capture
+ * before it exists, the batch is searched query by query. Same answers. */
 int ch_query_batch(ch_t *ch, const uint32_t *src, const uint32_t *dst, uint64_t k,
                    uint32_t *dist_out, uint32_t *settled_out, void *stream);
 

@@ -106,6 +106,15 @@ void dev_release(void *p, size_t cls) {
     c.bytes += cls;
 }
 
+size_t dev_available() {
+    size_t free_bytes = 0, total = 0;
+    CH_CUDA_TRY(cudaMemGetInfo(&free_bytes, &total));
+    const int dev = current_device();
+    if (dev < 0) return free_bytes;
+    std::lock_guard<std::mutex> lock(g_cache_mu);
+    return free_bytes + g_cache[dev].bytes;
+}
+
 size_t dev_trim() {
     const int dev = current_device();
     if (dev < 0) return 0;

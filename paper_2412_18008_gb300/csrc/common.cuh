@@ -65,9 +65,11 @@ bool inject_alloc_failure();
 // the block's class size, which dev_release needs. A block may be released
 // only once the device no longer uses it. dev_trim waits for the device and
 // frees the cached blocks of the current device (returns their bytes).
+// dev_available: bytes that are free on the current device or in its cache.
 void *dev_alloc(size_t bytes, size_t *got);
 void dev_release(void *p, size_t cls);
 size_t dev_trim();
+size_t dev_available();
 
 // A device array owned by the library (memory from dev_alloc). Releasing it
 // (destruction, alloc, move-assignment) hands the block back to the cache,

@@ -624,6 +624,11 @@ bool query_labels_prepare(ch_s *h, uint64_t k) {
         return false;
     }
     const size_t n = h->n;
+    const size_t entries = std::max<size_t>(2 * n * HL_AVG, 1u << 16);
+    // Labels only make the batch faster, and the arena is far larger than the
+    // hierarchy: it takes at most a quarter of what the device has left, so that
+    // what the caller allocates next fits as it would with searches.
+    if (entries * sizeof(uint2) > dev_available() / 4) return false;
     try {
         DevBuf<uint2> arena;
         DevBuf<uint32_t> label;
@@ -636,7 +641,7 @@ bool query_labels_prepare(ch_s *h, uint64_t k) {
         label.alloc(4 * n);
         mark.alloc(2 * n);
         cursor.alloc(1);
-        arena.alloc(std::max<size_t>(2 * n * HL_AVG, 1u << 16));
+        arena.alloc(entries);
         h->hl_label = std::move(label);
         h->hl_mark = std::move(mark);
         h->hl_list = std::move(list);
