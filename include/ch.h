@@ -336,7 +336,11 @@ int ch_load(const char *path, ch_t **out);
  * threads, small_first 1, stall 1 and delta = 128 x its weight scale (the
  * median weight of 1024 evenly spaced E_up edges; delta = 0 when it has a
  * core, whose searches outgrow the shared tables anyway). Every
- * configuration gives the same answers and search-space sizes. */
+ * configuration gives the same answers and search-space sizes. It is that of
+ * batches whose queries are searched in blocks of this kind: batches of at
+ * most one query an SM have a kernel of their own, batches answered through
+ * hub labels (ch_query_batch) use it for what the labels leave over, and
+ * hierarchies with a large core and no core table do not use it. */
 #define CH_QUERY_BLOCK_FLAT 0u
 #define CH_QUERY_WARP_FLAT 1u
 typedef struct {
@@ -352,7 +356,8 @@ int ch_get_query_config(const ch_t *ch, ch_query_config_t *cfg);
 
 /* Times each configuration on `sample` seeded uniform random queries (a
  * warm-up run, then one run timed with CUDA events on `stream`) and keeps
- * the fastest for the handle. ms_out (or NULL) receives the
+ * the fastest for the handle; whatever the sample's size, its queries are
+ * searched, not answered through labels. ms_out (or NULL) receives the
  * CH_QUERY_AUTOTUNE_CONFIGS times: index 4 * small_first +
  * 2 * (layout == WARP_FLAT) + (threads == 256) without stalling or delta;
  * then 8 + 2 * small_first + (threads == 256) for the warp layout with
@@ -368,8 +373,9 @@ int ch_query_autotune(ch_t *ch, uint64_t sample, uint32_t seed, void *stream,
  * Builds `graph` once per (hop limit, witness_route_deg) pair of the two
  * lists, other parameters as in `params` (NULL: defaults), and times each
  * build (ch_stats_t.build_ms) and a batch of `sample` seeded uniform random
- * queries on it (a warm-up run, then one run timed with CUDA events on
- * params->stream). A candidate's cost is
+ * queries on it, answered as ch_query_batch answers a batch of that size (a
+ * warm-up run, then one run timed with CUDA events on params->stream). A
+ * candidate's cost is
  *     build_ms + query_ms * queries_per_build / sample;
  * the cheapest hierarchy is returned in *out and the others are freed.
  * results (or NULL) receives one row per candidate, hop limits outer, and

@@ -137,7 +137,8 @@ void query_work(ch_s *h, cudaStream_t st, uint64_t out[2]);
 // Whether nearly all searches of the handle's configuration fit 2^11-slot tables
 // (a sample of seeded random pairs, run on `st` and waited for the first time).
 bool query_fits_small(ch_s *h, cudaStream_t st);
-// Device time (ms) of a batch of `sample` seeded random queries (after one warm-up batch).
+// Device time (ms) of a batch of `sample` seeded random queries, answered as any
+// batch of that size is (after one warm-up batch).
 double query_time_sample(ch_s *h, uint64_t sample, uint32_t seed, cudaStream_t st);
 ch_query_graph_s *query_graph_create(ch_s *h, const uint32_t *src, const uint32_t *dst, uint64_t k,
                                      uint32_t *dist_out);

@@ -900,9 +900,9 @@ double query_time_sample(ch_s *h, uint64_t sample, uint32_t seed, cudaStream_t s
     float ms = 0;
     cudaError_t e = cudaSuccess;
     try {
-        query_batch(h, s, t, sample, out, nullptr, st, true);  // warm-up
+        query_batch(h, s, t, sample, out, nullptr, st);  // warm-up
         CH_CUDA_TRY(cudaEventRecord(e0, st));
-        query_batch(h, s, t, sample, out, nullptr, st, true);
+        query_batch(h, s, t, sample, out, nullptr, st);
         CH_CUDA_TRY(cudaEventRecord(e1, st));
         CH_CUDA_TRY(cudaEventSynchronize(e1));
         e = cudaEventElapsedTime(&ms, e0, e1);
