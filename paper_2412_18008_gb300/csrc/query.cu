@@ -186,26 +186,24 @@ __device__ void dense_query(QDSmem &q, const QArgs &a, const QDense &dn, uint32_
         uint32_t *ncnt = &q.cnt3[(lvl + 1) % 3];
         uint32_t lmf = INF, lmb = INF;  // least labels this thread queues
         for (uint32_t t0 = 0; t0 < nfront; t0 += QD_THREADS) {
+            // Barriers keep this part of a tile, which reads labels and takes
+            // vertices out of the queue, apart from the relaxations of this
+            // tile and of the one before: a label read here is current, and one
+            // lowered later finds the vertex's bit clear and queues it again.
             const uint32_t fi = t0 + tid;
             const uint32_t ent = fi < nfront ? __ldcg(cur + fi) : 0;
             const uint32_t x = ent & 0x7FFFFFFFu, dir = ent >> 31;
             bool ok = fi < nfront && x < a.n;
             if (fi < nfront && !ok) atomicOr(a.err, QERR_BOUND);
             uint32_t *dist = dir ? db : df;
-            uint32_t lab = ok ? __ldcg(dist + x) : INF;
+            const uint32_t lab = ok ? __ldcg(dist + x) : INF;
             bool keep = false;
             if (PRUNE) {
                 const bool drop = ok && (lab >= mu0 || (x >= a.core_first &&
                                                         sat_add(lab, dir ? minf : minb) >= mu0));
                 keep = ok && !drop && lab > (dir ? thrb : thrf);
                 if (drop) {
-                    // a label lowered meanwhile is queued again
                     atomicAnd(&queued[x], ~(1u << dir));
-                    const uint32_t now = __ldcg(dist + x);
-                    if (now < lab) {
-                        lab = now;
-                        if (!(atomicOr(&queued[x], 1u << dir) & (1u << dir))) keep = true;
-                    }
                     ok = false;
                 }
                 const uint32_t m = __ballot_sync(FULL, keep);
@@ -225,10 +223,7 @@ __device__ void dense_query(QDSmem &q, const QArgs &a, const QDense &dn, uint32_
             }
             uint32_t b = 0, cnt = 0;
             if (ok) {
-                // out of the queue first, then its label: one lowered after
-                // this read queues the vertex again
                 atomicAnd(&queued[x], ~(1u << dir));
-                lab = __ldcg(dist + x);
                 const uint32_t *off = dir ? a.dn_off : a.up_off;
                 b = off[x];
                 const uint32_t e = off[x + 1];
