@@ -3164,13 +3164,14 @@ void Builder::run_rounds() {
         finish_row();  // the round before
         const Ctl c = *hctl;
         const uint32_t nF = c.nF, nS2 = c.nS2, nAnext = c.nAnext;
-        last_nS = c.nS;
+        if (nA) last_nS = c.nS;
         // overflow of the score phase's middle tier decides the next two phases'
-        // launches: a few sources are left to the dense tier
+        // launches: a few sources are left to the dense tier (a round without
+        // a score phase says nothing)
         if (skip_mid) {
             --skip_mid;  // the middle tier is tried again in the end
-        } else {
-            if (use_big && nA && c.nOvf1 > 64 && 8ull * c.nOvf1 > 5ull * (score_direct ? c.nS : c.nOvf)) skip_mid = 16;
+        } else if (nA) {
+            if (use_big && c.nOvf1 > 64 && 8ull * c.nOvf1 > 5ull * (score_direct ? c.nS : c.nOvf)) skip_mid = 16;
             use_big = (use_big ? c.nOvf1 : c.nOvf2) > 4;
         }
         if (nF == 0) {
