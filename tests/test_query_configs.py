@@ -48,6 +48,17 @@ def test_every_configuration_gives_the_oracle_answers(geo, cfg):
     assert np.array_equal(d[idx], O.dijkstra_pairs(g, s[idx], t[idx]))
 
 
+@pytest.mark.parametrize("cfg", [(lay, thr, sf, 0, 0) for sf in (0, 1) for lay in (0, 1) for thr in (128, 256)]
+                         + [(1, thr, sf, 1, 0) for sf in (0, 1) for thr in (128, 256)] + DELTA_CASES)
+def test_every_configuration_searches_a_batch_below_the_label_line(geo, cfg):
+    g, gch, och = geo
+    gch.set_query_config(*cfg)
+    s, t = I.random_pairs(g.n, 15_000, seed=89)
+    gch.query_work()
+    assert np.array_equal(gch.query(s, t), och.query(s, t))
+    assert gch.query_work()[0] > 10 * s.size  # a search a query; labels expand each vertex twice at most
+
+
 def test_configurations_on_a_dense_random_digraph():
     g = I.random_digraph(1500, 9000, 1, 1000, seed=83)
     gch = _ch().CH.build(g, hop_limit=4)
