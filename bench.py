@@ -752,8 +752,10 @@ def main():
             if qcfg is not None:
                 h.set_query_config(*qcfg)
             e1.record(stream)
+            batch0 = ch.kernel_launches()
             if not args.build_only:
                 h.query_batch_raw(s_d.data_ptr(), t_d.data_ptr(), nq, out_d.data_ptr(), None, sp)
+            batch_launches = ch.kernel_launches() - batch0
             e2.record(stream)
         stream.synchronize()
         step_ms.append(e0.elapsed_time(e2))
@@ -822,9 +824,9 @@ def main():
         # with stalling each expansion also reads the other CSR's two offsets
         stall = bool(qcfg[3]) if qcfg else False
         l2_record = None
-        # batches of this size, on a hierarchy without a core, are answered
-        # through hub labels (ch_query_batch), not by a search a query
-        labels = nq >= 1 << 14 and nq * nq >= 6400 * stats["n"] and not stats["core_vertices"]
+        # a batch of searches is at most three launches (two table sizes and the
+        # dense kernel); one answered through hub labels has one a level
+        labels = batch_launches > 4
         if not labels and args.workload == "geo1M" and qcfg is not None and tuple(qcfg) == QUERY_L2_CONFIG:
             l2_peak = l2_read_gbs(dev)
             l2_gbs = QUERY_L2_BYTES_PER_QUERY * nq / (mean_query * 1e-3) / 1e9

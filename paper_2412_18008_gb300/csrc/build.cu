@@ -29,8 +29,9 @@
 // scan by itself), each allowed to start while the one before it ends
 // (programmatic dependent launch), step times stamped by the kernels instead
 // of event records between them, and the host's one read handed over by the
-// last kernel it depends on. 1M-vertex geometric graph, 215 rounds: 94.0 -> 54.8
-// ms; 64 x 64 grid, 43 rounds: 12.7 -> 6.1 ms.
+// last kernel it depends on. With the middle witness tier and summed counters,
+// 1M-vertex geometric graph, 215 rounds: 94 -> 57 ms (48 now, with block warps
+// sharing short lists); 64 x 64 grid, 43 rounds: 12.7 -> 6.2 ms.
 //
 // The witness distance is d_H(a, b), the least weight of a walk a -> b with
 // at most H edges in the round's overlay (INF if none); a candidate
@@ -2515,6 +2516,10 @@ __global__ void k_insert(Dev d, const uint4 *rec, const uint8_t *flag, uint32_t 
     }
 }
 
+// --------------------------------------------------------------------------
+// Postprocess: rank by (level, score, id) and the rank-ordered CSRs
+// --------------------------------------------------------------------------
+
 __global__ void k_rank_keys(const uint32_t *level, const int32_t *P, uint32_t n, uint64_t *keys,
                             uint32_t *vals) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
@@ -2935,8 +2940,8 @@ void Builder::normalise(const ch_graph_t *g) {
 template <int MODE>
 void Builder::witness(const uint32_t *Sl, const uint32_t *nS_dev, uint32_t nS_max, uint32_t expected, uint32_t r,
                       unsigned long long *ts) {
-    // the tiers' work counters (work .. work4, nOvf, nOvf1, nOvf2) are zeroed
-    // by k_round_begin / k_contract_begin before each phase
+    // the tiers' work counters (work .. work4, nOvf, nOvf1, nOvf2) are zero: the
+    // round before ended with round_begin, k_contract_prep with phase_begin
     WArgs a;
     a.d = d;
     a.S = Sl;
@@ -3000,18 +3005,19 @@ void Builder::launch_witness(const WArgs &a, uint32_t nS_max, uint32_t expected)
                        a, mid);
             ++h->witness_launches;
         } else {
-        if (!use_big) {
-            mid.out = ovf2.ptr;
-            mid.out_cnt = &c->nOvf2;
-        }
-        launch_pdl(k_witness_block<MODE, FEAT, MidSmem<MODE>>, few ? std::min(mid_blocks_few, (int)expected + 16) : mid_blocks,
-                   few ? WM_THREADS_FEW : WM_THREADS_MANY, sizeof(MidSmem<MODE>), st, a, mid);
-        ++h->witness_launches;
-        if (use_big) {
-            launch_pdl(k_witness_block<MODE, FEAT, BigSmem<MODE>>, big_blocks, WB_THREADS, sizeof(BigSmem<MODE>), st,
-                       a, big);
+            if (!use_big) {
+                mid.out = ovf2.ptr;
+                mid.out_cnt = &c->nOvf2;
+            }
+            launch_pdl(k_witness_block<MODE, FEAT, MidSmem<MODE>>,
+                       few ? std::min(mid_blocks_few, (int)expected + 16) : mid_blocks,
+                       few ? WM_THREADS_FEW : WM_THREADS_MANY, sizeof(MidSmem<MODE>), st, a, mid);
             ++h->witness_launches;
-        }
+            if (use_big) {
+                launch_pdl(k_witness_block<MODE, FEAT, BigSmem<MODE>>, big_blocks, WB_THREADS, sizeof(BigSmem<MODE>),
+                           st, a, big);
+                ++h->witness_launches;
+            }
         }
     }
     launch_pdl(k_witness_dense<MODE, FEAT>, dense.nslots, 256, 0, st, a, dense);

@@ -334,10 +334,11 @@ __device__ __forceinline__ void cp_async_wait() {
 // parameters and streams both operands through a ring of four chunks of 64
 // samples (asynchronous copies, 80 KB, so that two blocks share an SM and the
 // 160 blocks of 8192 samples run at once); a thread holds 2 x 2 sums of W2
-// (or 4 x 2 of W1), so that its chains hide each other's latency. Bound by the
-// chain of 512 dependent multiply-adds and the staging. (One block a slice, a
-// thread a parameter reading global memory: 16 blocks and 470 us for 8192
-// samples; this takes 22.)
+// (or 4 x 2 of W1), so that its chains hide each other's latency. 22 us for 8192
+// samples, about one block of four warps an SM: the chain of 512 dependent
+// multiply-adds is about 1 us of it, the rest the latency of the staged chunks
+// and of the shared-memory reads that so few warps cannot hide. (One block a
+// slice, a thread a parameter reading global memory: 16 blocks and 470 us.)
 __global__ void __launch_bounds__(TRG_THREADS)
 k_train_grad_part(const float *x, uint64_t b0, uint32_t bsz, const float *h1, const float *h2,
                   const float *g1, const float *g2, const float *dy, float *part) {

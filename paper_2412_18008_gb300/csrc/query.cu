@@ -378,8 +378,9 @@ __global__ void __launch_bounds__(QD_THREADS) k_query_dense(QArgs a, QDense dn) 
 // are dealt to 32 warps, most of which hold one or two, and each row's lanes
 // read its stall edges and its out-edges together, without the scans and owner
 // searches of flattened rows. An entry found stalled drops the out-edges it has
-// read. Geometric graph of 1M vertices: 69 us a query alone, 114 for 152 at
-// once, against 122 and 216 by the launches that larger batches take. (Rows
+// read. Geometric graph of 1M vertices, back to back: 63 us for a query, 114 for
+// 152, against 122 and 216 by the launches that larger batches take (a query
+// that is waited for takes 80 us, launch and wait included). (Rows
 // flattened over the whole block: 80 and 133 us. Whole rows in the blocks of
 // 256 threads that larger batches use, several rows a warp: slower, 302 us for
 // 777 queries against 254.)

@@ -25,7 +25,7 @@ def _graph(name):
         return I.geometric_knn_graph(14_000, seed=200)
     wide = I.random_digraph(4_000, 14_000, 1, 1000, seed=201)
     if name == "wide_many":
-        return I.random_digraph(12_000, 42_000, 1, 1000, seed=203)
+        return I.random_digraph(12_000, 60_000, 1, 1000, seed=203)
     if name == "wide":  # most balls outgrow the middle tier
         return wide
     return _union(I.geometric_knn_graph(12_000, seed=202), wide)
