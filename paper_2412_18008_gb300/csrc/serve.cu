@@ -316,7 +316,8 @@ __global__ void __launch_bounds__(QB_THREADS, TB == 11 ? 6 : 1) k_serve(SvArgs a
     uint32_t seen = 0;                     // thread 0: entry (ticket + 1) whose descriptor s_* hold
     uint64_t seen_pos = 0;
     const unsigned long long long_ns = SV_CLAIM_NS * gridDim.x;
-    unsigned long long mean_ns = long_ns, begin_ns = 0;  // thread 0: time of a pair (one position first), this one's start
+    // thread 0: time of a pair (just short until the first one), this one's start
+    unsigned long long mean_ns = long_ns - 1, begin_ns = 0;
     while (true) {
         __syncthreads();
         // Thread 0 takes the next published pool position. A position is
